@@ -45,10 +45,11 @@ typedef enum {
   HZ_ENOMEM = 2,      /* device allocation failed */
   HZ_ECUDA = 3,       /* a CUDA runtime call or kernel launch failed */
   HZ_ENOCONV = 4,     /* max_pc reached before the tolerance (results are filled) */
-  HZ_ETIMEOUT = 5,    /* a bounded device wait gave up: a grid barrier of the persistent
+  HZ_ETIMEOUT = 5,    /* a bounded device wait gave up: a copy that the complex64 forward
+                         stencil waits for did not land, or a grid barrier of the persistent
                          bottom-solve kernel (opt-in: environment HZ_PERSISTENT=1 when the
                          handle is created; all its blocks are co-resident by a cooperative
-                         launch) did not release within about a second.  The
+                         launch) did not release, within about a second.  The
                          kernel finishes without waiting, its results are invalid, and the
                          next helmholtz_solve or helmholtz_adjoint_grad on the handle
                          returns this status (threegrid_precond, being asynchronous, does
@@ -175,6 +176,8 @@ hz_status hz_set_params(hz_handle* h, const hz_params* params);
  *                is written (saturating at 255; 1 everywhere is an exact cover).
  *   blocks       HOST, or NULL: blocks per right-hand side (the fused
  *                reductions keep one partial sum per block).
+ *                The complex128 launch's; violations covers the complex64
+ *                launch of a forward application too (it tiles differently).
  *   violations   HOST: tiles whose threads would write outside the grid, use a
  *                row form that omits PML terms present at a written node, or
  *                repeat / overrun a block id.  0 for a valid layout.
@@ -232,7 +235,8 @@ hz_status iofd_jacobi(hz_handle* h, int level, int op, int precision, int nsweep
  *                  r must not alias g or x.
  *   norm2_dev      DEVICE double, nrhs values out.
  * Limits: nrhs <= 64 and (blocks per rhs of the launch that runs -- forward
- * or adjoint, which tile differently; hz_layout_check reports both) * nrhs
+ * or adjoint, which tile differently; hz_layout_check reports both, and the
+ * complex128 launch counts for either precision) * nrhs
  * <= 65536; larger problems return HZ_EINVAL with a message.  The first call on a device looks
  * up the array's device address (cudaGetSymbolAddress) and should come before
  * any stream capture.  Every call shares the one array: calls that overlap on

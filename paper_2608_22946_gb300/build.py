@@ -17,11 +17,12 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libhz.so")
-# (source, extra flags, object): the forward stencil source is compiled once
-# per (precision, mode) part so that its kernels build in parallel
+# (source, extra flags, object): the forward stencil sources are compiled once
+# per mode so that their kernels build in parallel
 SOURCES = [("hz_stencil.cu", [], "hz_stencil.o"), ("hz_vec.cu", [], "hz_vec.o"), ("hz_solver.cu", [], "hz_solver.o"),
            ("hz_fwd_gather.cu", [], "hz_fwd_gather.o"), ("hz_block.cu", [], "hz_block.o")] + [
-    ("hz_fwd.cu", [f"-DHZ_FWD_PART={k}"], f"hz_fwd_{k}.o") for k in range(6)]
+    ("hz_fwd.cu", [f"-DHZ_FWD_PART={k}"], f"hz_fwd_{k}.o") for k in range(5)] + [
+    ("hz_march.cu", [f"-DHZ_MARCH_PART={k}"], f"hz_march_{k}.o") for k in range(4)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I" + INCLUDE, "-I" + CSRC]

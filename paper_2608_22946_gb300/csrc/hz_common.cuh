@@ -136,6 +136,10 @@ struct LevelView {
   const cx<R>* eps[3][2];
   // precombined coefficient polynomials of this level (layout in hz_fwd.cuh)
   const R* ctab;
+  // the same for the single-precision kernels of hz_march.cuh (null for double)
+  const R* mtab;
+  int nsub;                       // parts per segment of their table S
+  int strip[4];                   // their PML strip tiles: w, h below / above the core, w, h beside it
   int plain_lo[3], plain_hi[3];
   R inv_ell2;                     // 1 / ell^2
   int zblock;                     // planes per CTA of the forward stencil (0: heuristic)

@@ -53,6 +53,7 @@ struct StencilCall {
   // y + rhs * ystride + (z - zr0) * plane (strides 0: N)
   int zr0 = 0, zr1 = 0, xz0 = 0;
   long long xstride = 0, ystride = 0;
+  int* err = nullptr;  // device flag set when a bounded wait of the kernel gave up
 };
 
 template <class R>
@@ -65,8 +66,10 @@ template <class R, int MODE>
 void fwd_init_attrs();
 // Smallest z-block (planes per CTA) of a stencil launch.
 constexpr int kMinZblock = 2;
-// (level 0 runs the accumulation-form kernels of hz_fwd.cuh, levels 1 and 2 the
-// gather-form kernels of hz_fwd_gather.cu; each has its own launch layout)
+// (in double precision level 0 runs the accumulation-form kernels of hz_fwd.cuh,
+// levels 1 and 2 the gather-form kernels of hz_fwd_gather.cu; single precision
+// runs hz_march.cuh on every level, small grids the gather form; each has its own
+// launch layout)
 long long stencil_blocks_per_rhs(int level, int nx, int ny, int nz, const int* plain_lo, const int* plain_hi,
                                  int nrhs, int zblock = 0, int zblock_f = 0);
 // Blocks per right-hand side of an adjoint stencil launch (zblock > 0 forces it).
@@ -98,8 +101,37 @@ void launch_block_gram(const BlockCols& X, const BlockCols& Y, double* partial, 
 template <class R>
 void launch_block_update(const BlockCols& X, cx<R>* Y, int q, const double* C, double beta, cudaStream_t s);
 void block_init_attrs();
+namespace march {
+// forward stencil in single precision, every level (hz_march.cuh)
+// Small grids take the gather-form kernels of hz_fwd_gather.cu, on every level:
+// their marches are a few planes long, and the longer prologue (tables, the
+// copies' latency) and larger code of the march cost more than its steady state
+// gains, the more so the more the mode stages.  In a graph, us, gather / march:
+//   apply B     39^3 4.3 / 5.6, 73^3 8.2 / 8.7, 77^3 10.0 / 10.0, 89^3 13.1 / 13.1
+//               (A 13.1 / 12.1), 97^3 16.2 / 16.1, 113^3 21.7 / 20.6, 129^3 31 / 25.7
+//   residual    97^3 25.6 / 27.9, 113^3 38.2 / 34.8; two right-hand sides 41.1 /
+//               49.3 and 61 / 53.6
+//   J_2         97^3 20.0 / 24.8, 113^3 28.5 / 30.8, 129^3 41.6 / 37.8; two
+//               right-hand sides 97^3 37.4 / 38.9, 113^3 51 / 47.2
+inline bool takes(int mode, int nx, int ny, int nz, int nrhs) {
+  const long long n = (long long)nx * ny * nz;
+  if (mode == M_RESID) return n >= 1LL << 20;
+  if (mode == M_J2) return n * (nrhs > 1 ? 2 : 1) >= 1LL << 21;
+  return n >= 1LL << 19;
+}
+void launch(const StencilCall<float>& c, int mode, int opk, cudaStream_t s);
+void init_attrs();
+// Tiles of the PML strips of a grid (LevelView::strip); searched once per level.
+void strips(int nx, int ny, const int* plo, const int* phi, int* strip);
+long long blocks_per_rhs(int nx, int ny, int nz, const int* plain_lo, const int* plain_hi, int nrhs, int zblock,
+                         int zblock_f, const int* strip = nullptr);
+long long replay_layout(int nx, int ny, int nz, const int* plo, const int* phi, int op, int nrhs, int zblock,
+                        int zblock_f);
+}  // namespace march
+
 namespace gather {
-// forward stencil of the coarse levels (hz_fwd_gather.cu)
+// forward stencil of the coarse levels in double precision and of small grids in
+// single precision (hz_fwd_gather.cu)
 template <class R>
 void launch_fwd_gather(const StencilCall<R>& c, int mode, int op, cudaStream_t s);
 long long gather_blocks_per_rhs(int nx, int ny, int nz, const int* plain_lo, const int* plain_hi, int nrhs,

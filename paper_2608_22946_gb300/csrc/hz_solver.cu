@@ -26,6 +26,7 @@
 
 #include "hz.h"
 #include "hz_fwd.cuh"
+#include "hz_march.cuh"
 #include "hz_kernels.h"
 
 using namespace hz;
@@ -97,6 +98,8 @@ struct Level {
   cx<float>* eps_f[3][2] = {};
   double* ctab_d = nullptr;
   float* ctab_f = nullptr;
+  int strip[4] = {};        // PML strip tiles of the single-precision forward kernels
+  float* mtab_f = nullptr;  // tables of the single-precision forward kernels (hz_march.cuh)
   int plain_lo[3] = {}, plain_hi[3] = {};
   // 1/diag of the operator each Jacobi map of Algorithm 1 uses on this level
   // ([0]: A_L, [1]: B_L); complex64 set at creation, complex128 on first use
@@ -141,6 +144,7 @@ struct hz_handle {
   double* tab_d = nullptr;
   float* tab_f = nullptr;
   int nseg = 0;
+  int nsub = 4;  // parts per segment of the single-precision kernels' table S
   double ds = 0;
   Work<float> wf;
   Work<double> wd;
@@ -161,6 +165,7 @@ struct hz_handle {
   double *s_nrm = nullptr, *s_root = nullptr, *s_inv = nullptr;
   std::map<std::tuple<int, int, int, const void*, void*>, std::pair<cudaGraphExec_t, unsigned long long>> graphs;
   double t_setup = 0;
+  bool tuned_c64 = false;  // z-blocks were timed in single precision
   bool use_graphs = true;
   // the bottom solve C_4h as one persistent cooperative kernel (forward, m_4h = 4,
   // two Jacobi sweeps; opt-in through HZ_PERSISTENT=1 at creation); its
@@ -184,6 +189,7 @@ template <> struct Sel<float> {
   static const cx<float>* dinv(const Level& L, bool shifted) { return L.dinv_f[shifted ? 1 : 0]; }
   static const cx<float>* eps(const Level& L, int a, int s) { return L.eps_f[a][s]; }
   static const float* ctab(const Level& L) { return L.ctab_f; }
+  static const float* mtab(const Level& L) { return L.mtab_f; }
   static constexpr int prec = HZ_C64;
 };
 template <> struct Sel<double> {
@@ -195,6 +201,7 @@ template <> struct Sel<double> {
   static const cx<double>* dinv(const Level& L, bool shifted) { return L.dinv_d[shifted ? 1 : 0]; }
   static const cx<double>* eps(const Level& L, int a, int s) { return L.eps_d[a][s]; }
   static const double* ctab(const Level& L) { return L.ctab_d; }
+  static const double* mtab(const Level&) { return nullptr; }
   static constexpr int prec = HZ_C128;
 };
 
@@ -356,6 +363,123 @@ void build_coef_tables(const std::vector<double>& coef, const double* rows, int 
   }
 }
 
+// Tables of the single-precision forward kernels (hz_march.cuh): the same
+// functions, in the coordinate u = eta / ds - k measured in segments from the
+// node k ds, and the cubics of nsub parts of each segment.
+struct MarchFns {
+  Poly a4, a5, Lm[4], Mm[4], Qm[4], Cm[4];  // on one segment; Cm times ell^2
+};
+MarchFns march_fns(const std::vector<double>& coef, const double* rows, int K, double ds, int k) {
+  MarchFns F;
+  Poly P[kNumFn];
+  for (int f = 0; f < kNumFn; ++f) {
+    if (k < K - 1) {
+      P[f] = poly_shift(&coef[((size_t)k * kNumFn + f) * 4], 3, k * ds - rows[k * 17]);
+    } else {
+      P[f] = Poly{};
+      P[f][0] = rows[(K - 1) * 17 + (f < 5 ? 1 + f : 11 + (f - 5))];
+    }
+    double sc = 1.0;
+    for (int j = 0; j < 6; ++j, sc *= ds) P[f][j] *= sc;  // u in segments
+  }
+  auto shell = [&](int a, Poly* w) {  // weights (f_a, f_{a+1} / 6, f_{a+2} / 12, rest / 8)
+    w[0] = P[a];
+    w[1] = poly_lin(0.0, P[a + 1], 1.0 / 6.0);
+    w[2] = poly_lin(0.0, P[a + 2], 1.0 / 12.0);
+    w[3] = poly_add(poly_add(poly_lin(0.125, P[a], -0.125), P[a + 1], -0.125), P[a + 2], -0.125);
+  };
+  F.a4 = P[3];
+  F.a5 = P[4];
+  F.Lm[0] = poly_lin(0.0, F.a4, 6.0);
+  F.Lm[1] = poly_add(F.a5, F.a4, -1.0);
+  F.Lm[2] = poly_add(poly_lin(0.5, F.a4, -0.5), F.a5, -1.0);
+  F.Lm[3] = poly_add(poly_lin(-0.75, F.a4, 0.75), F.a5, 0.75);
+  shell(0, F.Mm);
+  shell(5, F.Qm);
+  const double q = 4.0 * M_PI * M_PI * ds * ds;  // kappa^2 = (2 pi ds)^2 (k + u)^2
+  for (int m = 0; m < 4; ++m) F.Cm[m] = poly_add(F.Lm[m], poly_mul_quad(F.Mm[m], q * k * k, 2.0 * q * k, q), -1.0);
+  return F;
+}
+double poly_at(const Poly& p, double u) {
+  double s = 0.0;
+  for (int j = 5; j >= 0; --j) s = s * u + p[j];
+  return s;
+}
+// power basis (in x = nsub u - b) of the cubic through p at the Chebyshev nodes of part b
+std::array<double, 4> part_cubic(const Poly& p, int nsub, int b) {
+  double x[4], f[4];
+  std::array<double, 4> c{};
+  for (int i = 0; i < 4; ++i) {
+    x[i] = 0.5 - 0.5 * std::cos(M_PI * (2 * i + 1) / 8.0);
+    f[i] = poly_at(p, (b + x[i]) / nsub);
+  }
+  for (int s = 1; s < 4; ++s)  // Newton's divided differences, then the power basis
+    for (int i = 3; i >= s; --i) f[i] = (f[i] - f[i - 1]) / (x[i] - x[i - s]);
+  c[0] = f[3];
+  for (int s = 2; s >= 0; --s) {
+    for (int j = 3; j >= 1; --j) c[j] = c[j - 1] - x[s] * c[j];
+    c[0] = f[s] - x[s] * c[0];
+  }
+  return c;
+}
+// parts per segment that the cubics need (kSubTol)
+int march_parts(const std::vector<double>& coef, const double* rows, int K, double ds) {
+  constexpr double mult[4] = {1, 6, 12, 8};  // nodes of each shell
+  for (int nsub = 1;; nsub *= 2) {
+    if (2 * nsub * (K - 1) > march::kMaxParts) return nsub;
+    double worst = 0.0;
+    for (int k = 0; k < K - 1; ++k) {
+      const MarchFns F = march_fns(coef, rows, K, ds, k);
+      for (int b = 0; b < nsub; ++b) {
+        double err = 0.0, scale = 0.0;
+        for (int m = 0; m < 4; ++m) {
+          const std::array<double, 4> c = part_cubic(F.Cm[m], nsub, b);
+          for (int i = 0; i <= 16; ++i) {
+            const double x = i / 16.0, ex = poly_at(F.Cm[m], (b + x) / nsub);
+            err = std::max(err, mult[m] * std::fabs(c[0] + x * (c[1] + x * (c[2] + x * c[3])) - ex));
+            scale = std::max(scale, mult[m] * std::fabs(ex));
+          }
+        }
+        worst = std::max(worst, err / scale);
+      }
+    }
+    if (worst <= march::kSubTol) return nsub;
+  }
+}
+
+void build_march_tables(const std::vector<double>& coef, const double* rows, int K, double ds, double ell, int nsub,
+                        std::vector<float>& out) {
+  const int ns = K;
+  out.assign((size_t)march::mt_size(ns), 0.f);
+  const double inv_l2 = 1.0 / (ell * ell);
+  const size_t oF = (size_t)march::kMtC * ns, oQ = oF + (size_t)march::kMtF * ns;
+  for (int k = 0; k < ns; ++k) {
+    const MarchFns F = march_fns(coef, rows, K, ds, k);
+    for (int m = 0; m < 4; ++m) {
+      for (int j = 0; j < 6; ++j) out[(size_t)k * march::kMtC + 4 * j + m] = (float)(inv_l2 * F.Cm[m][j]);
+      for (int j = 0; j < 4; ++j) {
+        out[oF + (size_t)k * march::kMtF + 6 * j + 2 + m] = (float)F.Mm[m][j];
+        out[oQ + (size_t)k * march::kMtQ + 4 * j + m] = (float)F.Qm[m][j];
+      }
+    }
+    for (int j = 0; j < 4; ++j) {
+      out[oF + (size_t)k * march::kMtF + 6 * j] = (float)F.a4[j];
+      out[oF + (size_t)k * march::kMtF + 6 * j + 1] = (float)F.a5[j];
+    }
+    for (int b = 0; b < (k < K - 1 ? nsub : 1); ++b)
+      for (int m = 0; m < 6; ++m) {
+        const Poly& p = m < 4 ? F.Cm[m] : (m == 4 ? F.a4 : F.a5);
+        std::array<double, 4> c;
+        if (k == K - 1)  // beyond the clamp the functions are quadratics
+          for (int j = 0; j < 4; ++j) c[j] = p[j] * std::pow(1.0 / nsub, j);
+        else c = part_cubic(p, nsub, b);
+        const size_t o = (size_t)march::mt_off_S(ns) + march::kMtS * ((size_t)nsub * k + b);
+        for (int j = 0; j < 4; ++j)
+          out[m < 4 ? o + 4 * j + m : o + 16 + 2 * j + m - 4] = (float)((m < 4 ? inv_l2 : 1.0) * c[j]);
+      }
+  }
+}
+
 template <class R>
 LevelView<R> view(hz_handle* H, int L) {
   const Level& lv = H->lev[L];
@@ -375,9 +499,14 @@ LevelView<R> view(hz_handle* H, int L) {
     v.plain_hi[a] = lv.plain_hi[a];
   }
   v.ctab = Sel<R>::ctab(lv);
+  v.mtab = Sel<R>::mtab(lv);
+  v.nsub = H->nsub;
+  for (int i = 0; i < 4; ++i) v.strip[i] = lv.strip[i];
   v.inv_ell2 = (R)(1.0 / (lv.ell * lv.ell));
   v.zblock = lv.zblock;
   v.zblock_f = lv.zblock_f;
+  // z-blocks tuned on the complex64 kernels say nothing about the FP64-bound ones
+  if (sizeof(R) == sizeof(double) && H->tuned_c64) v.zblock = v.zblock_f = 0;
   return v;
 }
 template <class R>
@@ -431,6 +560,7 @@ StencilCall<R> call(hz_handle* H, int L, bool shifted, int nrhs) {
   c.side = H->side;
   c.fork = H->ev_fork;
   c.join = H->ev_join;
+  c.err = H->bot_err;
   return c;
 }
 
@@ -799,14 +929,20 @@ void level_dims(const hz_grid& g, int L, Level& lv) {
   const int nn[3] = {g.nx / f, g.ny / f, g.nz / f};
   std::vector<std::complex<double>> ab, ac;
   for (int a = 0; a < 3; ++a) pml_axis(nn[a], lv.n_pml, g.gamma_max, ab, ac, lv.plain_lo[a], lv.plain_hi[a]);
+  march::strips(lv.nx, lv.ny, lv.plain_lo, lv.plain_hi, lv.strip);
 }
 
 // Block partial sums of one fused stencil reduction (forward or adjoint
 // launch) on level lv with nrhs right-hand sides, at the z-blocks it will run.
-long long resid_blocks(const Level& lv, int level, int nrhs, bool adjoint) {
+// (The forward count is that of the complex128 launch; fwd_blocks_c64 has the complex64 one.)
+long long resid_blocks(const Level& lv, int level, int nrhs, bool adjoint, int zblock, int zblock_f) {
   return adjoint ? adj_blocks_per_rhs(lv.nx, lv.ny, lv.nz, nrhs)
-                 : stencil_blocks_per_rhs(level, lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nrhs, lv.zblock,
-                                          lv.zblock_f);
+                 : stencil_blocks_per_rhs(level, lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nrhs, zblock, zblock_f);
+}
+
+long long fwd_blocks_c64(const Level& lv, int nrhs) {
+  return march::blocks_per_rhs(lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nrhs, lv.zblock, lv.zblock_f,
+                                lv.strip);
 }
 
 // Per-block partial sums: the vector reductions use at most 1216 x 56, a fused
@@ -819,6 +955,9 @@ size_t red_partial_size(const Level* lev, int nrhs) {
                                                1, kMinZblock, kMinZblock);
     const long long a = adj_blocks_per_rhs(lev[L].nx, lev[L].ny, lev[L].nz, 1, kMinZblock);
     m = std::max(m, (size_t)std::max(f, a));
+    for (int r = 1; r <= 2; ++r)  // (one and two right-hand sides per block tile differently)
+      m = std::max(m, (size_t)march::blocks_per_rhs(lev[L].nx, lev[L].ny, lev[L].nz, lev[L].plain_lo, lev[L].plain_hi,
+                                                    r, kMinZblock, kMinZblock));
   }
   return m * nrhs;
 }
@@ -831,7 +970,7 @@ void plan_all(hz_handle* H, bool count_only) {
     Level& lv = H->lev[L];
     level_dims(H->g, L, lv);
     lv.kap_d = al.get<double>(lv.N);
-    lv.kap_f = al.get<float>(lv.N);
+    lv.kap_f = al.get<float>(lv.N + 1);  // the forward kernels read one element past a row's end
     const int nn[3] = {lv.nx, lv.ny, lv.nz};
     for (int a = 0; a < 3; ++a) {
       lv.abar_d[a] = al.get<cx<double>>(nn[a]);
@@ -845,15 +984,17 @@ void plan_all(hz_handle* H, bool count_only) {
     }
     lv.ctab_d = al.get<double>((size_t)kCtPerSeg * (kMaxSeg + 1));
     lv.ctab_f = al.get<float>((size_t)kCtPerSeg * (kMaxSeg + 1));
+    lv.mtab_f = al.get<float>((size_t)march::mt_size(kMaxSeg + 1));
   }
-  H->lev[0].dinv_f[0] = al.get<cx<float>>(H->lev[0].N);
-  H->lev[1].dinv_f[1] = al.get<cx<float>>(H->lev[1].N);
-  H->lev[2].dinv_f[1] = al.get<cx<float>>(H->lev[2].N);
+  H->lev[0].dinv_f[0] = al.get<cx<float>>(H->lev[0].N + 1);
+  H->lev[1].dinv_f[1] = al.get<cx<float>>(H->lev[1].N + 1);
+  H->lev[2].dinv_f[1] = al.get<cx<float>>(H->lev[2].N + 1);
   H->tab_d = al.get<double>((size_t)kMaxSeg * kNumFn * 4);
   H->tab_f = al.get<float>((size_t)kMaxSeg * kNumFn * 4);
   const int nr = H->max_nrhs;
   H->red_partial = al.get<double>(red_partial_size(H->lev, nr));
   H->red_count = al.get<unsigned>(nr);
+  H->bot_err = al.get<int>(1);
   H->cgs_skip = al.get<int>(nr);
   H->s_nrm = al.get<double>(nr);
   H->s_root = al.get<double>(nr);
@@ -966,7 +1107,11 @@ void autotune_zblocks(hz_handle* H) {
       return ms;
     };
     const bool split =
-        stencil_blocks_per_rhs(L, lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr, kMinZblock, 64) !=
+        sizeof(R) == sizeof(float)
+            ? march::blocks_per_rhs(lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr, kMinZblock, 64, lv.strip) !=
+                  march::blocks_per_rhs(lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr, kMinZblock, kMinZblock,
+                                        lv.strip)
+            : stencil_blocks_per_rhs(L, lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr, kMinZblock, 64) !=
         stencil_blocks_per_rhs(L, lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr, kMinZblock, kMinZblock);
     for (int pass = 0; pass < (split ? 2 : 1); ++pass) {
       float best_t = 1e30f;
@@ -1434,8 +1579,8 @@ SolveOut solve_c128(hz_handle* H, const cx<double>* b, cx<double>* x, int nrhs, 
   return o;
 }
 
-// A grid-barrier wait of the persistent bottom solve that gave up sets a
-// device flag (the kernel then finishes without waiting, its results
+// A bounded wait that gave up (a copy of the forward stencil, a grid barrier of
+// the persistent bottom solve) sets a device flag (the kernel then finishes without waiting, its results
 // invalid); the synchronous entry points read and clear it.
 void check_bottom_err(hz_handle* H) {
   if (!H->bot_err) return;
@@ -1445,7 +1590,7 @@ void check_bottom_err(hz_handle* H) {
   if (e) {
     HZ_CK(cudaMemsetAsync(H->bot_err, 0, sizeof(int), H->st));
     HZ_CK(cudaStreamSynchronize(H->st));
-    throw Fail{HZ_ETIMEOUT, "a grid-barrier wait of the persistent bottom solve gave up; the results are invalid"};
+    throw Fail{HZ_ETIMEOUT, "a bounded wait of a kernel gave up; the results are invalid"};
   }
 }
 
@@ -1610,6 +1755,7 @@ hz_status hz_create(const hz_grid* grid, const double* c_dev, const hz_params* p
     auto t0 = std::chrono::steady_clock::now();
     plan_all(H, false);
     HZ_CK(cudaMemsetAsync(H->red_count, 0, sizeof(unsigned) * max_nrhs, H->st));
+    HZ_CK(cudaMemsetAsync(H->bot_err, 0, sizeof(int), H->st));
     {
       // opt-in: on the 289^3 benchmark the ten grid barriers cost more than the
       // launch gaps they replace (15.0 against 14.2-14.5 ms per preconditioner call)
@@ -1622,10 +1768,8 @@ hz_status hz_create(const hz_grid* grid, const double* c_dev, const hz_params* p
       }
       if (H->coop_bottom) {
         H->bot_bar = H->al.get<unsigned>(2);
-        H->bot_err = H->al.get<int>(1);
         H->bot_partial_f = H->al.get<double>(gather::bottom_partial_doubles<float>(max_nrhs));
         H->bot_partial_d = H->al.get<double>(gather::bottom_partial_doubles<double>(max_nrhs));
-        HZ_CK(cudaMemsetAsync(H->bot_err, 0, sizeof(int), H->st));
       }
     }
     std::vector<double> coef;
@@ -1633,6 +1777,7 @@ hz_status hz_create(const hz_grid* grid, const double* c_dev, const hz_params* p
     build_table(table_host, table_rows, coef, ds);
     H->nseg = table_rows - 1;
     H->ds = ds;
+    H->nsub = march_parts(coef, table_host, table_rows, ds);
     std::vector<float> coef_f(coef.begin(), coef.end());
     HZ_CK(cudaMemcpyAsync(H->tab_d, coef.data(), coef.size() * sizeof(double), cudaMemcpyHostToDevice, H->st));
     HZ_CK(cudaMemcpyAsync(H->tab_f, coef_f.data(), coef_f.size() * sizeof(float), cudaMemcpyHostToDevice, H->st));
@@ -1671,6 +1816,9 @@ hz_status hz_create(const hz_grid* grid, const double* c_dev, const hz_params* p
         std::vector<float> ct_f(ct_s.begin(), ct_s.end());
         HZ_CK(cudaMemcpy(lv.ctab_d, ct_d.data(), ct_d.size() * sizeof(double), cudaMemcpyHostToDevice));
         HZ_CK(cudaMemcpy(lv.ctab_f, ct_f.data(), ct_f.size() * sizeof(float), cudaMemcpyHostToDevice));
+        std::vector<float> mt;
+        build_march_tables(coef, table_host, table_rows, ds, lv.ell, H->nsub, mt);
+        HZ_CK(cudaMemcpy(lv.mtab_f, mt.data(), mt.size() * sizeof(float), cudaMemcpyHostToDevice));
       }
       launch_setup_kappa<double>(c_dev, H->g.nx + 1, H->g.ny + 1, H->g.nz + 1, H->g.n_pml, f, H->g.omega, lv.ell,
                                  lv.kap_d, H->st);
@@ -1682,6 +1830,7 @@ hz_status hz_create(const hz_grid* grid, const double* c_dev, const hz_params* p
     HZ_LAUNCHED();
     if (H->p.precision == HZ_C128) prepare_dinv_double(H);
     if (H->p.autotune) {
+      H->tuned_c64 = H->p.precision == HZ_C64;
       if (H->p.precision == HZ_C64) autotune_zblocks<float>(H);
       else autotune_zblocks<double>(H);
     }
@@ -2100,7 +2249,8 @@ extern "C" hz_status iofd_residual_static(hz_handle* H, int level, int op, int p
     const Level& lv = H->lev[level];
     const bool adj0 = (op == HZ_OP_A_ADJ || op == HZ_OP_B_ADJ);
     // partial sums of the launch that will run (forward and adjoint tile differently)
-    const long long need = resid_blocks(lv, level, nrhs, adj0) * nrhs;
+    const LevelView<double> lvd = view<double>(H, level);
+    const long long need = resid_blocks(lv, level, nrhs, adj0, lvd.zblock, lvd.zblock_f) * nrhs;
     HZ_REQUIRE(need <= kResidStaticPartials,
                "grid too large for the static scratch (" + std::to_string(need) + " block partial sums > " +
                    std::to_string(kResidStaticPartials) + ")");
@@ -2119,8 +2269,12 @@ extern "C" hz_status iofd_residual_static(hz_handle* H, int level, int op, int p
       c.x = (const cx<float>*)x;
       c.g = (const cx<float>*)g;
       c.y = (cx<float>*)r;
-      c.red = red;
+      // the limit above is counted on the complex128 launch in either precision; a
+      // complex64 launch of more blocks leaves its norm to a pass of at most 608
+      const bool fused = adj || fwd_blocks_c64(lv, nrhs) * nrhs <= kResidStaticPartials;
+      if (fused) c.red = red;
       launch_stencil<float>(c, M_RESID, OP_AB, adj, st);
+      if (!fused) launch_norm2<float>(c.y, (int)lv.N, nrhs, red, st);
     } else {
       StencilCall<double> c = call<double>(H, level, shifted, nrhs);
       c.x = (const cx<double>*)x;

@@ -25,25 +25,15 @@
 namespace hz {
 
 // the forward kernels are instantiated in hz_fwd.cu
-extern template void launch_fwd<float, M_APPLY>(const StencilCall<float>&, int, cudaStream_t);
-extern template void launch_fwd<float, M_RESID>(const StencilCall<float>&, int, cudaStream_t);
-extern template void launch_fwd<float, M_J2>(const StencilCall<float>&, int, cudaStream_t);
-extern template void launch_fwd<float, M_JSWEEP>(const StencilCall<float>&, int, cudaStream_t);
 extern template void launch_fwd<double, M_APPLY>(const StencilCall<double>&, int, cudaStream_t);
 extern template void launch_fwd<double, M_RESID>(const StencilCall<double>&, int, cudaStream_t);
 extern template void launch_fwd<double, M_J2>(const StencilCall<double>&, int, cudaStream_t);
 extern template void launch_fwd<double, M_JSWEEP>(const StencilCall<double>&, int, cudaStream_t);
-extern template void launch_fwd<float, M_AWIN>(const StencilCall<float>&, int, cudaStream_t);
 extern template void launch_fwd<double, M_AWIN>(const StencilCall<double>&, int, cudaStream_t);
-extern template void fwd_init_attrs<float, M_APPLY>();
-extern template void fwd_init_attrs<float, M_RESID>();
-extern template void fwd_init_attrs<float, M_J2>();
-extern template void fwd_init_attrs<float, M_JSWEEP>();
 extern template void fwd_init_attrs<double, M_APPLY>();
 extern template void fwd_init_attrs<double, M_RESID>();
 extern template void fwd_init_attrs<double, M_J2>();
 extern template void fwd_init_attrs<double, M_JSWEEP>();
-extern template void fwd_init_attrs<float, M_AWIN>();
 extern template void fwd_init_attrs<double, M_AWIN>();
 
 constexpr int TX = 32, TY = 8, NT = TX * TY;
@@ -287,22 +277,23 @@ void launch_stencil(const StencilCall<R>& c, int mode, int op, bool adjoint, cud
     k_j1<R><<<blocks, 256, 0, s>>>(c, adjoint ? 1 : 0);
     return;
   }
-  if (!adjoint && c.lv.level > 0) {
-    gather::launch_fwd_gather<R>(c, mode, op, s);
-    return;
-  }
   if (!adjoint) {
     const int opk = fwd_opk(c, op);
-    if (op == OP_Q) {
+    if constexpr (sizeof(R) == sizeof(float)) {
+      if (mode == M_AWIN || march::takes(mode, c.lv.nx, c.lv.ny, c.lv.nz, c.nrhs)) march::launch(c, mode, opk, s);
+      else gather::launch_fwd_gather(c, mode, op, s);
+    } else if (c.lv.level > 0) {
+      gather::launch_fwd_gather(c, mode, op, s);
+    } else if (op == OP_Q) {
       launch_fwd<R, M_APPLY>(c, opk, s);
-      return;
-    }
-    switch (mode) {
-      case M_APPLY: launch_fwd<R, M_APPLY>(c, opk, s); break;
-      case M_RESID: launch_fwd<R, M_RESID>(c, opk, s); break;
-      case M_J2: launch_fwd<R, M_J2>(c, opk, s); break;
-      case M_JSWEEP: launch_fwd<R, M_JSWEEP>(c, opk, s); break;
-      case M_AWIN: launch_fwd<R, M_AWIN>(c, opk, s); break;
+    } else {
+      switch (mode) {
+        case M_APPLY: launch_fwd<R, M_APPLY>(c, opk, s); break;
+        case M_RESID: launch_fwd<R, M_RESID>(c, opk, s); break;
+        case M_J2: launch_fwd<R, M_J2>(c, opk, s); break;
+        case M_JSWEEP: launch_fwd<R, M_JSWEEP>(c, opk, s); break;
+        case M_AWIN: launch_fwd<R, M_AWIN>(c, opk, s); break;
+      }
     }
   } else {
     if (op == OP_Q) {
@@ -346,14 +337,19 @@ long long adj_blocks_per_rhs(int nx, int ny, int nz, int nrhs, int zblock) {
 // saturating at 255.
 long long replay_fwd_layout(int level, int nx, int ny, int nz, const int* plo, const int* phi, int op, int nrhs,
                             int zblock, int zblock_f, unsigned char* counts, long long* blocks) {
-  if (level > 0) return gather::replay_gather_layout(nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f, counts, blocks);
+  // the single-precision launch has a layout of its own (march, small grids gather)
+  long long single = march::replay_layout(nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f);
+  if (level == 0 && !march::takes(M_J2, nx, ny, nz, 1))
+    single += gather::replay_gather_layout(nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f, nullptr, nullptr);
+  if (level > 0)
+    return single + gather::replay_gather_layout(nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f, counts, blocks);
   const bool ab = op == OP_AB;
   const int zb = zblock > 0 ? zblock : choose_zblock(nx, ny, nz, nrhs);
   const FwdPlan p = plan_layout(nx, ny, nz, plo, phi, ab, zb, zblock_f);
   const long long nblk = p.blocks();
   if (blocks) *blocks = nblk;
   std::vector<unsigned char> seen((size_t)nblk, 0);
-  long long bad = 0;
+  long long bad = single;
   auto plain_x = [&](int x) { return x >= plo[0] && x <= phi[0]; };
   auto plain_y = [&](int y) { return y >= plo[1] && y <= phi[1]; };
   // one block of a tile shape (npx columns per thread, txt x tyt threads)
@@ -461,15 +457,11 @@ void init_kernel_attributes() {
   set_adj_attr<double, M_J2, OP_AB>();
   set_adj_attr<double, M_JSWEEP, OP_AB>();
   set_adj_attr<double, M_APPLY, OP_Q>();
-  fwd_init_attrs<float, M_APPLY>();
-  fwd_init_attrs<float, M_RESID>();
-  fwd_init_attrs<float, M_J2>();
-  fwd_init_attrs<float, M_JSWEEP>();
+  march::init_attrs();
   fwd_init_attrs<double, M_APPLY>();
   fwd_init_attrs<double, M_RESID>();
   fwd_init_attrs<double, M_J2>();
   fwd_init_attrs<double, M_JSWEEP>();
-  fwd_init_attrs<float, M_AWIN>();
   fwd_init_attrs<double, M_AWIN>();
 }
 
