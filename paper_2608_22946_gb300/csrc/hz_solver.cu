@@ -611,7 +611,7 @@ void jacobi(hz_handle* H, int L, bool shifted, bool adj, const cx<R>* g, cx<R>* 
     return;
   }
   c.dinv = Sel<R>::dinv(H->lev[L], shifted);
-  HZ_REQUIRE(adj || c.dinv, "internal: Jacobi diagonal of this level/operator was not prepared");
+  HZ_REQUIRE(c.dinv, "internal: Jacobi diagonal of this level/operator was not prepared");
   if (nJ == 2) {
     c.x = g;
     c.y = y;

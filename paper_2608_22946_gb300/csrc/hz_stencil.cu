@@ -13,9 +13,6 @@
 // Coefficients are evaluated per row from kappa = k ell through the cubic
 // Hermite tables at eta* = min(kappa / 2 pi, 0.4) (Eq. iofd-clamped-coordinate).
 //
-// The adjoint kernel applies (H^H x)_i = sum_delta conj(H_{i+delta}(-delta)) x_{i+delta};
-// it needs the neighbours' own coefficients, which it evaluates once per
-// loaded node into shared memory.
 #include <algorithm>
 #include <cstdio>
 #include <vector>
@@ -40,176 +37,233 @@ constexpr int TX = 32, TY = 8, NT = TX * TY;
 constexpr int PW = TX + 2, PH = TY + 2, PLANE = PW * PH;
 
 // ----------------------------------------------------------------------------
-// adjoint kernel: generic 27-neighbour gather with neighbour coefficients
+// adjoint kernel
 // ----------------------------------------------------------------------------
-template <int OP> struct AdjNP { static constexpr int v = 8; };
-template <> struct AdjNP<OP_Q> { static constexpr int v = 4; };
+// (H^H x)_i = sum_j conj(H_j(i - j)) x_j: every source node j spreads its own
+// row's weights.  With C_m the shell weights of row j, t_0..t_2 its transverse
+// weights and eps the PML factors, node j is turned once into u_m = conj(C_m) x
+// (m = 0..3) and, near a PML, v_c = t_c x (c = 0..2); plane q then contributes
+//   to its own rows   c(u_0) + e(u_1) + k(u_2),
+//   to rows q +- 1    c(u_1) + e(u_2) + k(u_3)
+// (c, e, k: centre, face and corner sums over the in-plane neighbours), and each
+// stretched axis adds the same sums of the v's along it,
+//   conj(eps+(j)) from the node at offset -1, conj(eps-(j)) from that at +1,
+//   -conj(eps+ + eps-) from the row's own position.
+// A block of 32 x 8 columns marches in z: each plane's nodes with their halo are
+// loaded one plane ahead, turned into the u's and v's in shared memory (two
+// buffers, one barrier per plane) and summed; a column keeps the partial sums of
+// two rows.  Evaluating the weights once per node instead of once per neighbour
+// (27 complex coefficients per output node) is what it gains: bound by issue in
+// single precision and by the FP64 rate in double.
+constexpr int kAdjF = 7;  // fields in shared memory: u_0..u_3, v_0..v_2
+template <class R>
+struct AdjSmem {
+  static constexpr size_t o_tab = (size_t)2 * kAdjF * PLANE * sizeof(cx<R>);
+  static size_t bytes(int opk, int ns) {
+    return o_tab + sizeof(R) * (opk == OPK_Q ? (size_t)kCtQ : (size_t)(kCtCA + kCtK + kCtT)) * ns;
+  }
+};
 
-template <class R, int MODE, int OP>
-__global__ void __launch_bounds__(NT) k_adj(StencilCall<R> a, int zblock, int tiles_x) {
-  constexpr int NP = AdjNP<OP>::v;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  cx<R>* sV = reinterpret_cast<cx<R>*>(smem_raw);            // [3][PLANE]
-  R* sP = reinterpret_cast<R*>(sV + 3 * PLANE);                // [3][PLANE][NP]
-  R* sTab = sP + 3 * PLANE * NP;                               // table
-  __shared__ double sRed[32];
+template <class R, int MODE, int OPK, bool GEN>
+__device__ __forceinline__ void adj_tile(const StencilCall<R>& a, unsigned char* smem, double* sRed, int zblock,
+                                         int tiles_x) {
+  constexpr bool Q = OPK == OPK_Q, B = OPK == OPK_B;
+  constexpr int NF = GEN ? kAdjF : 4;
   const LevelView<R>& L = a.lv;
+  cx<R>* sF = reinterpret_cast<cx<R>*>(smem);
+  R* sT = reinterpret_cast<R*>(smem + AdjSmem<R>::o_tab);
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-  for (int i = tid; i < a.tab.nseg * kNumFn * 4; i += NT) sTab[i] = a.tab.coef[i];
-  __syncthreads();
+  const int ns = a.tab.nseg + 1;
+  const R ds = a.tab.ds, inv_ds = a.tab.inv_ds;
+  if constexpr (Q) {
+    for (int i = tid; i < kCtQ * ns; i += NT) sT[i] = L.ctab[ct_off_Q(ns) + i];
+  } else {
+    for (int i = tid; i < (kCtCA + kCtK + kCtT) * ns; i += NT) sT[i] = L.ctab[i];
+  }
   const int rhs = blockIdx.x % a.nrhs, tile_x = blockIdx.x / a.nrhs;
   const int x0 = tile_x * TX, y0 = blockIdx.y * TY;
-  const int zb0 = blockIdx.z * zblock;
-  const int zb1 = min(zb0 + zblock, L.nz);
-  const long long N = L.N;
-  const long long plane_sz = (long long)L.nx * L.ny;
-  const cx<R>* X = a.x + rhs * N;
+  const int nx = L.nx, ny = L.ny, nz = L.nz;
+  const int zb0 = blockIdx.z * zblock, zb1 = min(zb0 + zblock, nz);
+  const int plane = nx * ny;
+  const cx<R>* X = a.x + rhs * L.N;
   const int gx = x0 + tx, gy = y0 + ty;
-  const bool active = (gx < L.nx) && (gy < L.ny);
-  const R inv_ell2 = L.inv_ell2;
-  const cx<R> shift = a.mass_shift;
-  const cx<R> cshift = conjc(shift);
-  const int nseg = a.tab.nseg;
-  const R ds = a.tab.ds, inv_ds = a.tab.inv_ds;
+  const bool active = gx < nx && gy < ny;
+  const R sigma = a.mass_shift.y, om = a.omega_j;
 
-  cx<R> abx[3], acx[3], aby[3], acy[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    int ix = min(max(gx + d - 1, 0), L.nx - 1), iy = min(max(gy + d - 1, 0), L.ny - 1);
-    abx[d] = L.abar[0][ix];
-    acx[d] = L.achk[0][ix];
-    aby[d] = L.abar[1][iy];
-    acy[d] = L.achk[1][iy];
+  // PML factors along x and y as this column meets them
+  const cx<R> zero = mkc<R>(0, 0);
+  cx<R> xm = zero, xp = zero, xc = zero, ym = zero, yp = zero, yc = zero;
+  bool xw = false, yw = false;
+  if constexpr (GEN) {
+    xw = x0 - 1 < L.plain_lo[0] || x0 + TX > L.plain_hi[0];
+    yw = y0 - 1 < L.plain_lo[1] || y0 + TY > L.plain_hi[1];
+    const int xi = min(gx, nx - 1), yi = min(gy, ny - 1);
+    xm = conjc(L.eps[0][0][max(xi - 1, 0)]);
+    xp = conjc(L.eps[0][1][min(xi + 1, nx - 1)]);
+    xc = conjc(L.eps[0][0][xi] + L.eps[0][1][xi]);
+    ym = conjc(L.eps[1][0][max(yi - 1, 0)]);
+    yp = conjc(L.eps[1][1][min(yi + 1, ny - 1)]);
+    yc = conjc(L.eps[1][0][yi] + L.eps[1][1][yi]);
   }
 
-  auto load = [&](int z, int slot) {
-    cx<R> abz = (z >= 0 && z < L.nz) ? L.abar[2][z] : mkc<R>(1, 0);
-    for (int i = tid; i < PLANE; i += NT) {
-      int ly = i / PW, lx = i - ly * PW;
-      int qx = x0 - 1 + lx, qy = y0 - 1 + ly;
-      bool in = (z >= 0) && (z < L.nz) && (qx >= 0) && (qx < L.nx) && (qy >= 0) && (qy < L.ny);
-      cx<R> v = mkc<R>(0, 0);
-      R prm[NP];
+  // this thread's (at most two) nodes of every halo plane, one plane ahead in registers
+  int go[2];
+  bool in[2];
 #pragma unroll
-      for (int j = 0; j < NP; ++j) prm[j] = 0;
-      if (in) {
-        long long off = (long long)z * plane_sz + (long long)qy * L.nx + qx;
-        v = X[off];
-        R kap = L.kappa[off];
-        if (OP == OP_Q) {
-          R b[3];
-          table_eval<R, 5, 3>(sTab, nseg, ds, inv_ds, eta_star(kap), b);
-          prm[0] = b[0];
-          prm[1] = b[1] * (R)(1.0 / 6.0);
-          prm[2] = b[2] * (R)(1.0 / 12.0);
-          prm[3] = ((R)1 - b[0] - b[1] - b[2]) * (R)0.125;
+  for (int j = 0; j < 2; ++j) {
+    const int li = tid + j * NT, ly = li / PW, lx = li - ly * PW;
+    const int qx = x0 - 1 + lx, qy = y0 - 1 + ly;
+    in[j] = li < PLANE && qx >= 0 && qx < nx && qy >= 0 && qy < ny;
+    go[j] = in[j] ? qy * nx + qx : 0;
+  }
+  cx<R> xv[2], dv[2];
+  R kv[2];
+  auto load = [&](int z) {
+    const bool zin = (unsigned)z < (unsigned)nz;
+    const long long o = zin ? (long long)z * plane : 0;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const bool ok = zin && in[j];
+      xv[j] = ok ? X[o + go[j]] : zero;
+      kv[j] = ok ? L.kappa[o + go[j]] : (R)0;
+      if constexpr (MODE == M_J2) dv[j] = ok ? a.dinv[o + go[j]] : zero;
+    }
+  };
+  auto stage = [&](int buf) {
+    cx<R>* F = sF + (size_t)buf * kAdjF * PLANE;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int li = tid + j * NT;
+      if (j && li >= PLANE) break;
+      cx<R> v = xv[j];
+      if constexpr (MODE == M_J2) v = cjmul(dv[j], v);  // y1 / omega = D^-H g
+      R u, C[4];
+      const int seg = seg_of(kv[j], ns, ds, inv_ds, u);
+      if constexpr (Q) {
+        horner_pm<R, 4, 3>(sT + seg * kCtQ, u, C);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) F[m * PLANE + li] = C[m] * v;
+      } else {
+        horner_pm<R, 4, 5>(sT + seg * kCtCA, u, C);
+        if constexpr (B) {
+          // conj(C - i sigma K) x
+          R Km[4];
+          horner_pm<R, 4, 5>(sT + ct_off_K(ns) + seg * kCtK, u, Km);
+#pragma unroll
+          for (int m = 0; m < 4; ++m) F[m * PLANE + li] = mkc<R>(C[m], sigma * Km[m]) * v;
         } else {
-          R av[5];
-          table_eval<R, 0, 5>(sTab, nseg, ds, inv_ds, eta_star(kap), av);
-          prm[0] = av[3];
-          prm[1] = av[4] * (R)0.25;
-          prm[2] = ((R)1 - av[3] - av[4]) * (R)0.25;
-          prm[3] = av[0];
-          prm[4] = av[1] * (R)(1.0 / 6.0);
-          prm[5] = av[2] * (R)(1.0 / 12.0);
-          prm[6] = ((R)1 - av[0] - av[1] - av[2]) * (R)0.125;
-          prm[7] = inv_ell2 * kap * kap;
-          if (MODE == M_J2) {
-            cx<R> sab = L.abar[0][qx] + L.abar[1][qy] + abz;
-            cx<R> D = inv_ell2 * ((R)2 * prm[0] * sab) - (prm[7] * prm[3]) * shift;
-            v = a.omega_j * cdiv(v, conjc(D));   // y1 = omega D^-H g
-          }
+#pragma unroll
+          for (int m = 0; m < 4; ++m) F[m * PLANE + li] = C[m] * v;
+        }
+        if constexpr (GEN) {
+          const RowT<R> t = eval_t(sT + ct_off_T(ns), seg, u);
+          F[4 * PLANE + li] = t.a4 * v;
+          F[5 * PLANE + li] = t.q5 * v;
+          F[6 * PLANE + li] = t.qb * v;
         }
       }
-      sV[slot * PLANE + i] = v;
-#pragma unroll
-      for (int j = 0; j < NP; ++j) sP[(slot * PLANE + i) * NP + j] = prm[j];
     }
   };
 
   R nrm2 = 0;
   const bool want_norm = MODE == M_RESID && a.red.out != nullptr;
-  load(zb0 - 1, (zb0 + 2) % 3);
-  load(zb0, zb0 % 3);
-  for (int z = zb0; z < zb1; ++z) {
-    load(z + 1, (z + 1) % 3);
+  cx<R> pa = zero, pb = zero;  // rows q - 1 and q so far
+  load(zb0 - 1);
+  __syncthreads();  // table
+  const int lc = (ty + 1) * PW + tx + 1;
+  for (int q = zb0 - 1; q <= zb1; ++q) {
+    const int buf = (q - zb0 + 1) & 1;
+    stage(buf);
+    if (q < zb1) load(q + 1);
     __syncthreads();
-    if (active) {
-      cx<R> abz[3], acz[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        int iz = min(max(z + d - 1, 0), L.nz - 1);
-        abz[d] = L.abar[2][iz];
-        acz[d] = L.achk[2][iz];
+    const cx<R>* F = sF + (size_t)buf * kAdjF * PLANE + lc;
+    auto face = [&](const cx<R>* f) { return (f[-1] + f[1]) + (f[-PW] + f[PW]); };
+    auto corner = [&](const cx<R>* f) { return (f[-PW - 1] + f[-PW + 1]) + (f[PW - 1] + f[PW + 1]); };
+    cx<R> p0 = F[0] + face(F + PLANE) + corner(F + 2 * PLANE);
+    cx<R> p1 = F[PLANE] + face(F + 2 * PLANE) + corner(F + 3 * PLANE);
+    cx<R> pm = p1, pp = p1;
+    if constexpr (GEN) {
+      const cx<R>*v0 = F + 4 * PLANE, *v1 = F + 5 * PLANE, *v2 = F + 6 * PLANE;
+      cx<R> s0 = zero, s1 = zero;
+      if (xw) {
+        auto X0 = [&](int d) { return v0[d] + (v1[d - PW] + v1[d + PW]); };
+        auto X1 = [&](int d) { return v1[d] + (v2[d - PW] + v2[d + PW]); };
+        s0 += xm * X0(-1) + xp * X0(1) - xc * X0(0);
+        s1 += xm * X1(-1) + xp * X1(1) - xc * X1(0);
       }
-      cx<R> acc = mkc<R>(0, 0);
-#pragma unroll
-      for (int dz = -1; dz <= 1; ++dz) {
-        const int slot = (z + dz + 3) % 3;
-#pragma unroll
-        for (int dy = -1; dy <= 1; ++dy) {
-#pragma unroll
-          for (int dx = -1; dx <= 1; ++dx) {
-            const int li = slot * PLANE + (ty + 1 + dy) * PW + (tx + 1 + dx);
-            const cx<R> v = sV[li];
-            const R* p = sP + li * NP;
-            const int sh = (dx != 0) + (dy != 0) + (dz != 0);
-            if (OP == OP_Q) {
-              acc += p[sh] * v;
-            } else {
-              // row j = i + delta reaches i at offset -delta
-              auto dval = [&](cx<R> ab, cx<R> ac, int off) -> cx<R> {
-                return off == 0 ? (R)(-2) * ab : (off > 0 ? ab + ac : ab - ac);
-              };
-              cx<R> st = p[(dy != 0) + (dz != 0)] * dval(abx[dx + 1], acx[dx + 1], -dx) +
-                         p[(dx != 0) + (dz != 0)] * dval(aby[dy + 1], acy[dy + 1], -dy) +
-                         p[(dx != 0) + (dy != 0)] * dval(abz[dz + 1], acz[dz + 1], -dz);
-              cx<R> coef = (-inv_ell2) * conjc(st) - (p[7] * p[3 + sh]) * cshift;
-              acc += coef * v;
-            }
-          }
-        }
+      if (yw) {
+        auto Y0 = [&](int d) { return v0[d] + (v1[d - 1] + v1[d + 1]); };
+        auto Y1 = [&](int d) { return v1[d] + (v2[d - 1] + v2[d + 1]); };
+        s0 += ym * Y0(-PW) + yp * Y0(PW) - yc * Y0(0);
+        s1 += ym * Y1(-PW) + yp * Y1(PW) - yc * Y1(0);
       }
-      const long long idx = (long long)z * plane_sz + (long long)gy * L.nx + gx;
-      cx<R> out;
-      if (MODE == M_APPLY) {
-        out = acc;
-      } else if (MODE == M_RESID) {
-        out = a.g[rhs * N + idx] - acc;
+      p0 += s0;
+      pm += s1;
+      pp += s1;
+      if ((unsigned)q < (unsigned)nz && (q < L.plain_lo[2] || q > L.plain_hi[2])) {
+        const cx<R> ep = L.eps[2][0][q], em = L.eps[2][1][q];
+        const cx<R> Z = v0[0] + face(v1) + corner(v2);
+        pp += conjc(ep) * Z;  // to row q + 1
+        pm += conjc(em) * Z;  // to row q - 1
+        p0 -= conjc(ep + em) * Z;
+      }
+    }
+    if (q > zb0 && active) {  // row q - 1 is complete
+      const cx<R> h = pa + pm;
+      const long long idx = (long long)(q - 1) * plane + gy * nx + gx;
+      cx<R> out = h;
+      if constexpr (MODE == M_RESID) {
+        out = a.g[rhs * L.N + idx] - h;
         if (want_norm) nrm2 += abs2(out);
-      } else {
-        const int li = (z % 3) * PLANE + (ty + 1) * PW + (tx + 1);
-        const R* p = sP + li * NP;
-        cx<R> sab = abx[1] + aby[1] + abz[1];
-        cx<R> Dh = conjc(inv_ell2 * ((R)2 * p[0] * sab) - (p[7] * p[3]) * shift);
-        if (MODE == M_J2) {
-          cx<R> g = X[idx];
-          out = sV[li] + a.omega_j * cdiv(g - acc, Dh);
-          if (a.base) out += a.base[rhs * N + idx];
-        } else {  // JSWEEP
-          out = sV[li] + a.omega_j * cdiv(a.g[rhs * N + idx] - acc, Dh);
+      } else if constexpr (MODE == M_J2) {
+        // with y1 = omega D^-H g and h = H^H y1 / omega:
+        // y1 + omega D^-H (g - H^H y1) = omega D^-H (2 g - omega h)
+        out = om * cjmul(a.dinv[idx], (R)2 * X[idx] - om * h);
+        if (a.base) out += a.base[rhs * L.N + idx];
+      } else if constexpr (MODE == M_JSWEEP) {
+        out = X[idx] + om * cjmul(a.dinv[idx], a.g[rhs * L.N + idx] - h);
+      }
+      a.y[rhs * L.N + idx] = out;
+    }
+    pa = pb + p0;
+    pb = pp;
+  }
+  if constexpr (MODE == M_RESID) {
+    if (a.red.out) {
+      double s = block_sum((double)nrm2, sRed, tid, NT);
+      const unsigned nblk = (unsigned)(tiles_x * gridDim.y * gridDim.z);
+      const unsigned bid = (unsigned)(tile_x + tiles_x * (blockIdx.y + gridDim.y * blockIdx.z));
+      if (tid == 0) a.red.partial[(size_t)rhs * nblk + bid] = s;
+      if (last_block_arrive(a.red.count + rhs, nblk, tid)) {
+        double t = 0.0;
+        for (unsigned b = tid; b < nblk; b += NT) t += __ldcg(a.red.partial + (size_t)rhs * nblk + b);
+        t = block_sum(t, sRed, tid, NT);
+        if (tid == 0) {
+          a.red.out[rhs] = t;
+          if (a.red.root) a.red.root[rhs] = sqrt(t);
+          if (a.red.inv_root) a.red.inv_root[rhs] = t > 1e-300 ? 1.0 / sqrt(t) : 0.0;
+          a.red.count[rhs] = 0;
         }
       }
-      a.y[rhs * N + idx] = out;
     }
-    __syncthreads();
   }
-  if (MODE == M_RESID && a.red.out) {
-    double s = block_sum((double)nrm2, sRed, tid, NT);
-    const unsigned nblk = (unsigned)(tiles_x * gridDim.y * gridDim.z);
-    const unsigned bid = (unsigned)(tile_x + tiles_x * (blockIdx.y + gridDim.y * blockIdx.z));
-    if (tid == 0) a.red.partial[(size_t)rhs * nblk + bid] = s;
-    if (last_block_arrive(a.red.count + rhs, nblk, tid)) {
-      double t = 0.0;
-      for (unsigned b = tid; b < nblk; b += NT) t += __ldcg(a.red.partial + (size_t)rhs * nblk + b);
-      t = block_sum(t, sRed, tid, NT);
-      if (tid == 0) {
-        a.red.out[rhs] = t;
-        if (a.red.root) a.red.root[rhs] = sqrt(t);
-        if (a.red.inv_root) a.red.inv_root[rhs] = t > 1e-300 ? 1.0 / sqrt(t) : 0.0;
-        a.red.count[rhs] = 0;
-      }
-    }
+}
+
+template <class R, int MODE, int OPK>
+__global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 1) k_adj(StencilCall<R> a, int zblock, int tiles_x) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double sRed[32];
+  if constexpr (OPK == OPK_Q) {
+    adj_tile<R, MODE, OPK, false>(a, smem_raw, sRed, zblock, tiles_x);
+  } else {
+    // a source node in the PML of any axis, the halo's included?
+    const LevelView<R>& L = a.lv;
+    const int x0 = (blockIdx.x / a.nrhs) * TX, y0 = blockIdx.y * TY;
+    const int zb0 = blockIdx.z * zblock, zb1 = min(zb0 + zblock, L.nz);
+    const bool plain = x0 - 1 >= L.plain_lo[0] && x0 + TX <= L.plain_hi[0] && y0 - 1 >= L.plain_lo[1] &&
+                       y0 + TY <= L.plain_hi[1] && zb0 - 1 >= L.plain_lo[2] && zb1 <= L.plain_hi[2];
+    if (plain) adj_tile<R, MODE, OPK, false>(a, smem_raw, sRed, zblock, tiles_x);
+    else adj_tile<R, MODE, OPK, true>(a, smem_raw, sRed, zblock, tiles_x);
   }
 }
 
@@ -248,16 +302,14 @@ static int adj_zblock(int nx, int ny, int nz, int nrhs) {
   return std::min(std::max(zb, 4), kMaxZb);
 }
 
-template <class R, int MODE, int OP>
+template <class R, int MODE, int OPK>
 static void launch_adj_t(const StencilCall<R>& c, cudaStream_t s) {
-  constexpr int NP = AdjNP<OP>::v;
   const LevelView<R>& L = c.lv;
   const int zb = adj_zblock(L.nx, L.ny, L.nz, c.nrhs);
   const int tiles_x = (L.nx + TX - 1) / TX;
   dim3 grid(tiles_x * c.nrhs, (L.ny + TY - 1) / TY, (L.nz + zb - 1) / zb);
-  size_t smem = 3 * PLANE * (sizeof(cx<R>) + NP * sizeof(R)) + kMaxSeg * kNumFn * 4 * sizeof(R);
   count_launch();
-  k_adj<R, MODE, OP><<<grid, dim3(TX, TY), smem, s>>>(c, zb, tiles_x);
+  k_adj<R, MODE, OPK><<<grid, dim3(TX, TY), AdjSmem<R>::bytes(OPK, c.tab.nseg + 1), s>>>(c, zb, tiles_x);
 }
 
 // forward operator kind of a call: A (real shell coefficients) unless the mass
@@ -296,15 +348,17 @@ void launch_stencil(const StencilCall<R>& c, int mode, int op, bool adjoint, cud
       }
     }
   } else {
-    if (op == OP_Q) {
-      launch_adj_t<R, M_APPLY, OP_Q>(c, s);
+    const int opk = fwd_opk(c, op);
+    if (opk == OPK_Q) {
+      launch_adj_t<R, M_APPLY, OPK_Q>(c, s);
       return;
     }
+    const bool b = opk == OPK_B;
     switch (mode) {
-      case M_APPLY: launch_adj_t<R, M_APPLY, OP_AB>(c, s); break;
-      case M_RESID: launch_adj_t<R, M_RESID, OP_AB>(c, s); break;
-      case M_J2: launch_adj_t<R, M_J2, OP_AB>(c, s); break;
-      case M_JSWEEP: launch_adj_t<R, M_JSWEEP, OP_AB>(c, s); break;
+      case M_APPLY: b ? launch_adj_t<R, M_APPLY, OPK_B>(c, s) : launch_adj_t<R, M_APPLY, OPK_A>(c, s); break;
+      case M_RESID: b ? launch_adj_t<R, M_RESID, OPK_B>(c, s) : launch_adj_t<R, M_RESID, OPK_A>(c, s); break;
+      case M_J2: b ? launch_adj_t<R, M_J2, OPK_B>(c, s) : launch_adj_t<R, M_J2, OPK_A>(c, s); break;
+      case M_JSWEEP: b ? launch_adj_t<R, M_JSWEEP, OPK_B>(c, s) : launch_adj_t<R, M_JSWEEP, OPK_A>(c, s); break;
     }
   }
 }
@@ -437,26 +491,29 @@ long long replay_adj_layout(int nx, int ny, int nz, int nrhs, int zblock, unsign
   return 0;
 }
 
-template <class R, int MODE, int OP>
+template <class R, int MODE, int OPK>
 static void set_adj_attr() {
-  constexpr int NP = AdjNP<OP>::v;
-  size_t smem = 3 * PLANE * (sizeof(cx<R>) + NP * sizeof(R)) + kMaxSeg * kNumFn * 4 * sizeof(R);
-  cudaFuncSetAttribute(k_adj<R, MODE, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_adj<R, MODE, OPK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)AdjSmem<R>::bytes(OPK, kMaxSeg + 1));
+}
+template <class R>
+static void set_adj_attrs() {
+  set_adj_attr<R, M_APPLY, OPK_A>();
+  set_adj_attr<R, M_RESID, OPK_A>();
+  set_adj_attr<R, M_J2, OPK_A>();
+  set_adj_attr<R, M_JSWEEP, OPK_A>();
+  set_adj_attr<R, M_APPLY, OPK_B>();
+  set_adj_attr<R, M_RESID, OPK_B>();
+  set_adj_attr<R, M_J2, OPK_B>();
+  set_adj_attr<R, M_JSWEEP, OPK_B>();
+  set_adj_attr<R, M_APPLY, OPK_Q>();
 }
 
 // Opt the stencil kernels into more than 48 KB of dynamic shared memory where
 // they need it.  Called before any launch and outside stream capture.
 void init_kernel_attributes() {
-  set_adj_attr<float, M_APPLY, OP_AB>();
-  set_adj_attr<float, M_RESID, OP_AB>();
-  set_adj_attr<float, M_J2, OP_AB>();
-  set_adj_attr<float, M_JSWEEP, OP_AB>();
-  set_adj_attr<float, M_APPLY, OP_Q>();
-  set_adj_attr<double, M_APPLY, OP_AB>();
-  set_adj_attr<double, M_RESID, OP_AB>();
-  set_adj_attr<double, M_J2, OP_AB>();
-  set_adj_attr<double, M_JSWEEP, OP_AB>();
-  set_adj_attr<double, M_APPLY, OP_Q>();
+  set_adj_attrs<float>();
+  set_adj_attrs<double>();
   march::init_attrs();
   fwd_init_attrs<double, M_APPLY>();
   fwd_init_attrs<double, M_RESID>();
