@@ -904,7 +904,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 2 : 1) k_bottom4h(BottomA
       sres[tid] = t;
     }
     __syncthreads();
-    if (tid == 0) gram_lsq_solve<KN>(sres, b.y + (size_t)rhs * b.ld * 2);
+    if (tid < 32) gram_lsq_solve<KN>(sres, b.y + (size_t)rhs * b.ld * 2, tid);
     __syncthreads();
   }
   grid_barrier(b.bar, gen, b.err, b.spins, b.extra);

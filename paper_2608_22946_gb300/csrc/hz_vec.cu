@@ -67,30 +67,56 @@ __global__ void __launch_bounds__(TRX * TRY) k_restrict(const cx<R>* __restrict_
   c[(long long)r * nxc * nyc * nzc + (Z * nyc + Y) * nxc + X] = acc;
 }
 
-// trilinear interpolation (Eq. prolongation) added to base: f = base + P c
+// trilinear interpolation (Eq. prolongation) added to base: f = base + P c.
+// A thread takes the up to 2 x 2 x 2 fine nodes of one coarse cell: eight coarse
+// loads for eight nodes instead of eight each (145^3: 21 us at one node per
+// thread, bound by those loads).
 template <class R>
 __global__ void __launch_bounds__(TRX * TRY) k_prolong_add(const cx<R>* __restrict__ c, const cx<R>* __restrict__ base,
                                                             cx<R>* __restrict__ f, int nxf, int nyf, int nzf) {
   const int nxc = (nxf - 1) / 2 + 1, nyc = (nyf - 1) / 2 + 1, nzc = (nzf - 1) / 2 + 1;
-  const int x = blockIdx.x * TRX + threadIdx.x, y = blockIdx.y * TRY + threadIdx.y;
-  if (x >= nxf || y >= nyf) return;
-  const int r = blockIdx.z / nzf, z = blockIdx.z - r * nzf;
-  const cx<R>* C = c + (long long)r * nxc * nyc * nzc;
-  // an odd fine index sits halfway between coarse nodes X0 and X0 + 1 (both
-  // inside the grid); an even one on X0 (the second term then has weight 0)
-  const int X0 = x >> 1, Y0 = y >> 1, Z0 = z >> 1;
-  const int ox = x & 1, oy = y & 1, oz = z & 1;
-  const R hx = ox ? (R)0.5 : (R)1, hy = oy ? (R)0.5 : (R)1, hz = oz ? (R)0.5 : (R)1;
-  const R gx = ox ? (R)0.5 : (R)0, gy = oy ? (R)0.5 : (R)0, gz = oz ? (R)0.5 : (R)0;
-  auto row = [&](int Z, int Y) {
-    const cx<R>* p = C + (Z * nyc + Y) * nxc + X0;
-    return hx * p[0] + gx * p[ox];
-  };
-  const cx<R> a0 = hy * row(Z0, Y0) + gy * row(Z0, Y0 + oy);
-  const cx<R> a1 = hy * row(Z0 + oz, Y0) + gy * row(Z0 + oz, Y0 + oy);
-  const cx<R> acc = hz * a0 + gz * a1;
-  const long long t = (long long)r * nxf * nyf * nzf + (z * nyf + y) * nxf + x;
-  f[t] = base ? base[t] + acc : acc;
+  const int X = blockIdx.x * TRX + threadIdx.x, Y = blockIdx.y * TRY + threadIdx.y;
+  if (X >= nxc || Y >= nyc) return;
+  const int r = blockIdx.z / nzc, Z = blockIdx.z - r * nzc;
+  const cx<R>* C = c + (long long)r * nxc * nyc * nzc + ((long long)Z * nyc + Y) * nxc + X;
+  // (an odd fine index is inside the grid where its right coarse neighbour is)
+  const bool ox = 2 * X + 1 < nxf, oy = 2 * Y + 1 < nyf, oz = 2 * Z + 1 < nzf;
+  const long long o = (long long)r * nxf * nyf * nzf + ((long long)(2 * Z) * nyf + 2 * Y) * nxf + 2 * X;
+  cx<R> v[2][2][2];  // coarse corners, then interpolated axis by axis
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const cx<R>* p = C + (k && oz ? nxc * nyc : 0) + (j && oy ? nxc : 0);
+      const cx<R> a = p[0], b = p[ox ? 1 : 0];
+      v[k][j][0] = a;
+      v[k][j][1] = (R)0.5 * a + (R)0.5 * b;
+    }
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) v[k][1][i] = (R)0.5 * v[k][0][i] + (R)0.5 * v[k][1][i];
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) v[1][j][i] = (R)0.5 * v[0][j][i] + (R)0.5 * v[1][j][i];
+  cx<R> b[2][2][2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const bool in = (!k || oz) && (!j || oy) && (!i || ox);
+        b[k][j][i] = base && in ? base[o + ((long long)k * nyf + j) * nxf + i] : mkc<R>(0, 0);
+      }
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if ((!k || oz) && (!j || oy) && (!i || ox)) f[o + ((long long)k * nyf + j) * nxf + i] = b[k][j][i] + v[k][j][i];
 }
 
 template <class R>
@@ -110,10 +136,10 @@ void launch_prolong_add(const cx<R>* coarse, const cx<R>* base, cx<R>* fine, int
                         cudaStream_t s) {
   const int nxc = (nxf - 1) / 2 + 1, nyc = (nyf - 1) / 2 + 1, nzc = (nzf - 1) / 2 + 1;
   const long long Nf = (long long)nxf * nyf * nzf, Nc = (long long)nxc * nyc * nzc;
-  const int chunk = std::max(1, 65535 / nzf);  // grid.z limit
+  const int chunk = std::max(1, 65535 / nzc);  // grid.z limit
   for (int r0 = 0; r0 < nrhs; r0 += chunk) {
     const int nr = std::min(chunk, nrhs - r0);
-    const dim3 grid((nxf + TRX - 1) / TRX, (nyf + TRY - 1) / TRY, nzf * nr);
+    const dim3 grid((nxc + TRX - 1) / TRX, (nyc + TRY - 1) / TRY, nzc * nr);
     count_launch();
     k_prolong_add<R><<<grid, dim3(TRX, TRY), 0, s>>>(coarse + r0 * Nc, base ? base + r0 * Nf : nullptr,
                                                       fine + r0 * Nf, nxf, nyf, nzf);
@@ -206,31 +232,32 @@ __device__ __forceinline__ void combine_partials(const double* partial, int nrhs
   __syncthreads();
 #pragma unroll 1
   for (int v = w; v < NV; v += VB / 32) {
+    // four independent chains: the loads' latency is paid once per 128 blocks
     if constexpr (sizeof(R) == sizeof(float)) {
       const float2* pp = reinterpret_cast<const float2*>(partial) + ((size_t)v * nrhs + rhs) * nblk;
-      dsf a{0.f, 0.f}, b{0.f, 0.f};
-      unsigned k = lane;
-      for (; k + 32 < nblk; k += 64) {  // two independent chains
-        const float2 q0 = __ldcg(pp + k), q1 = __ldcg(pp + k + 32);
-        a = ds_add(a, dsf{q0.x, q0.y});
-        b = ds_add(b, dsf{q1.x, q1.y});
+      dsf a[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = dsf{0.f, 0.f};
+      for (unsigned k = lane; k < nblk; k += 128) {
+        float2 q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = k + 32 * i < nblk ? __ldcg(pp + k + 32 * i) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = ds_add(a[i], dsf{q[i].x, q[i].y});
       }
-      if (k < nblk) {
-        const float2 q0 = __ldcg(pp + k);
-        a = ds_add(a, dsf{q0.x, q0.y});
-      }
-      const dsf t = ds_warp_sum(ds_add(a, b));
+      const dsf t = ds_warp_sum(ds_add(ds_add(a[0], a[1]), ds_add(a[2], a[3])));
       if (lane == 0) out[v] = (double)t.hi + (double)t.lo;
     } else {
       const double* pp = partial + ((size_t)v * nrhs + rhs) * nblk;
-      double a = 0.0, b = 0.0;
-      unsigned k = lane;
-      for (; k + 32 < nblk; k += 64) {
-        a += __ldcg(pp + k);
-        b += __ldcg(pp + k + 32);
+      double a[4] = {0.0, 0.0, 0.0, 0.0};
+      for (unsigned k = lane; k < nblk; k += 128) {
+        double q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = k + 32 * i < nblk ? __ldcg(pp + k + 32 * i) : 0.0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] += q[i];
       }
-      if (k < nblk) a += __ldcg(pp + k);
-      const double t = warp_sum(a + b);
+      const double t = warp_sum((a[0] + a[1]) + (a[2] + a[3]));
       if (lane == 0) out[v] = t;
     }
   }
@@ -725,9 +752,7 @@ void launch_lsq(const double* H, const double* beta, double* y, int m, int ld, i
 // ----------------------------------------------------------------------------
 // CA-GMRES bottom solve: Gram matrix of [p_0 .. p_s], CholQR, least squares
 // ----------------------------------------------------------------------------
-// The small Cholesky solve runs in one thread of the last block only: the
-// register cap (4 blocks per SM for the usual s = 4) sizes the streaming loop,
-// and whatever the solve does not fit in registers goes to local memory.
+// (the small solve runs in one warp of the last block: hz_gram_solve.cuh)
 template <class R, int KN>
 __global__ void __launch_bounds__(VB) k_gram(const cx<R>* __restrict__ P, long long pstride, int n,
                                                              double* y, int ld, Reduce red) {
@@ -760,9 +785,9 @@ __global__ void __launch_bounds__(VB) k_gram(const cx<R>* __restrict__ P, long l
   block_partials<R, NV>(acc, sm, red.partial, nrhs, rhs, nblk, blockIdx.x, tid);
   if (!last_block_arrive(red.count + rhs, nblk, tid)) return;
   combine_partials<R, NV>(red.partial, nrhs, rhs, nblk, sm, sres, tid);
-  if (tid != 0) return;
-  red.count[rhs] = 0;
-  gram_lsq_solve<KN>(sres, y + (size_t)rhs * ld * 2);
+  if (tid >= 32) return;
+  if (tid == 0) red.count[rhs] = 0;
+  gram_lsq_solve<KN>(sres, y + (size_t)rhs * ld * 2, tid);
 }
 
 template <class R>
