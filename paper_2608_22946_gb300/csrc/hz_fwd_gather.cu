@@ -32,13 +32,14 @@ constexpr int PW = TX + 2, PH = TY + 2, PLANE = PW * PH;
 template <int TX_, int TY_>
 struct TileShape {
   static constexpr int TXS = TX_, TYS = TY_, PWS = TX_ + 2, PLN = (TX_ + 2) * (TY_ + 2);
-  static_assert(TX_ * TY_ == NT, "one column per thread");
-  static_assert(PLN <= 2 * NT, "two load slots per thread");
+  static constexpr int NTH = TX_ * TY_;  // one column per thread
+  static_assert(PLN <= 2 * NTH, "two load slots per thread");
 };
 using TileSq = TileShape<TX, TY>;   // the PML-free rectangle; whole small grids
 using TileW = TileShape<64, 4>;     // PML strips below and above the rectangle (all x)
 using TileT = TileShape<4, 64>;     // PML strips left and right of it (its y range)
 using TileG = TileShape<16, 16>;    // whole small grids (coarse levels): fewer idle columns
+using TileS = TileShape<8, 8>;      // whole very small grids: many small blocks
 constexpr int NSTAGE = 6;   // shared-memory plane ring
 constexpr int PREF = 5;     // planes in flight ahead of the one consumed (NSTAGE - 1)
 
@@ -237,11 +238,11 @@ __host__ __device__ __forceinline__ FrameTile decode_frame(const TileMap& m, int
 template <class R, int MODE, int OP, int FORM, class TL>
 __device__ __forceinline__ void fwd_body(const StencilCall<R>& a, int zblock, int bz, const TileMap& tm, int rhs, int x0,
                                          int y0, int rx1, int ry1, unsigned bid, cx<R>* sX, cx<R>* sD, cx<R>* sY1,
-                                         const R* sTab, double* sRed, R (*sKc)[NT], cx<R> (*sGc)[NT]) {
-  constexpr int PWS = TL::PWS, PLN = TL::PLN;
+                                         const R* sTab, double* sRed, R (*sKc)[TL::NTH], cx<R> (*sGc)[TL::NTH]) {
+  constexpr int PWS = TL::PWS, PLN = TL::PLN, NT = TL::NTH;
   constexpr bool GEN = FORM != 0;
   const LevelView<R>& L = a.lv;
-  const int tid = threadIdx.y * TX + threadIdx.x;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   const int tx = tid % TL::TXS, ty = tid / TL::TXS;
   const int zb0 = bz * zblock;
   const int zb1 = min(zb0 + zblock, L.nz);
@@ -526,10 +527,39 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? (PATH == 0 ? 4 : 2) : 1) 
 }
 
 
+// A whole very small grid: 8 x 8 tiles of 64 threads.  A 256-thread tile puts a
+// 13^3 grid on 7 of 152 SMs, and in double precision a tile-plane takes an SM's two
+// FP64 lanes some 10 thousand cycles.
+template <class R, int MODE, int OP>
+__global__ void __launch_bounds__(TileS::NTH) k_fwd_small(StencilCall<R> a, int zblock, TileMap tm) {
+  constexpr int PL = TileS::PLN, NTS = TileS::NTH;
+  __shared__ __align__(16) cx<R> sX[NSTAGE * PL];
+  __shared__ __align__(16) cx<R> sD[(MODE == M_J2) ? NSTAGE * PL : 1];
+  __shared__ cx<R> sY1[(MODE == M_J2) ? PL : 1];
+  __shared__ __align__(16) R sTab[kMaxSeg * kNumFn * 4];
+  __shared__ R sKc[NSTAGE][NTS];
+  __shared__ cx<R> sGc[(MODE == M_RESID || MODE == M_JSWEEP) ? NSTAGE : 1][NTS];
+  __shared__ double sRed[32];
+  for (int i = threadIdx.x; i < a.tab.nseg * kNumFn * 4; i += NTS) sTab[i] = a.tab.coef[i];
+  const int rhs = blockIdx.x % a.nrhs, t = blockIdx.x / a.nrhs;
+  const unsigned bid = (unsigned)(t + tm.ntx * (blockIdx.y + gridDim.y * blockIdx.z));
+  const int x0 = t * TileS::TXS, y0 = (int)blockIdx.y * TileS::TYS;
+  const LevelView<R>& L = a.lv;
+  const bool plain = OP == OP_Q || (x0 >= L.plain_lo[0] && x0 + TileS::TXS - 1 <= L.plain_hi[0] &&
+                                    y0 >= L.plain_lo[1] && y0 + TileS::TYS - 1 <= L.plain_hi[1]);
+  if (plain)
+    fwd_body<R, MODE, OP, 0, TileS>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab,
+                                    sRed, sKc, sGc);
+  else if constexpr (OP != OP_Q)
+    fwd_body<R, MODE, OP, 2, TileS>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab,
+                                    sRed, sKc, sGc);
+}
+
 // ----------------------------------------------------------------------------
 // launcher
 // ----------------------------------------------------------------------------
 static int choose_zblock(int nx, int ny, int nz, int nrhs) {
+  if ((long long)nx * ny * nz <= kSmallNodes) return kMinZblock;
   long long tiles = (long long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY) * nrhs;
   // aim for about 4 waves of 2 CTAs on 152 SMs, with at least 4 planes per CTA
   long long want = 152LL * 2 * 4;
@@ -554,7 +584,8 @@ struct FwdPlan {
   int zb = 4, nzb = 1;     // whole grid or PML-free rectangle
   int zbf = 4, nzbf = 1;   // PML frame
   bool split = false;
-  int TXT = 1, TYT = 1;  // whole-grid tiling (16 x 16 for A/B, 32 x 8 for Q)
+  bool small = false;    // 8 x 8 whole-grid tiles
+  int TXT = 1, TYT = 1;  // whole-grid tiling (16 x 16 for A/B, 32 x 8 for Q, 8 x 8 when small)
   int RW = 0, RH = 0;    // 32 x 8 tiling of the PML-free rectangle
   TileMap frame;         // frame tiling (count = frame tiles per z-block)
   long long blocks() const {
@@ -573,6 +604,12 @@ static FwdPlan plan_layout(int nx, int ny, int nz, const int* plo, const int* ph
   const int px0 = std::max(plo[0], 0), px1 = std::min(phi[0], nx - 1);
   const int py0 = std::max(plo[1], 0), py1 = std::min(phi[1], ny - 1);
   p.split = (op == OP_AB) && (long long)nx * ny * nz >= kSplitNodes && px1 >= px0 && py1 >= py0;
+  p.small = (long long)nx * ny * nz <= kSmallNodes;
+  if (p.small) {
+    p.TXT = cdiv_i(nx, TileS::TXS);
+    p.TYT = cdiv_i(ny, TileS::TYS);
+    return p;
+  }
   if (!p.split) {
     if (op == OP_AB) {  // whole-grid launch of the A/B operators: 16 x 16 tiles
       p.TXT = (nx + TileG::TXS - 1) / TileG::TXS;
@@ -618,6 +655,10 @@ static void launch_fwd_t(const StencilCall<R>& c, cudaStream_t s) {
     tm.nblk_total = nblk_total;
     dim3 grid(p.TXT * c.nrhs, p.TYT, p.nzb);
     count_launch();
+    if (p.small) {
+      k_fwd_small<R, MODE, OP><<<grid, TileS::NTH, 0, s>>>(c, p.zb, tm);
+      return;
+    }
     k_fwd<R, MODE, OP, (OP == OP_Q) ? 0 : 2><<<grid, dim3(TX, TY), 0, s>>>(c, p.zb, tm);
     return;
   }
@@ -680,10 +721,11 @@ long long replay_gather_layout(int nx, int ny, int nz, const int* plo, const int
   const bool ab = op == OP_AB;
   auto plain_x = [&](int x) { return x >= plo[0] && x <= phi[0]; };
   auto plain_y = [&](int y) { return y >= plo[1] && y <= phi[1]; };
+  const int nth = p.small ? TileS::NTH : NT;
   auto cta = [&](int TXS, int x0, int y0, int rx1, int ry1, int form, int zbk, int bz, long long bid) {
     if (bid < 0 || bid >= nblk || seen[(size_t)bid]++) ++bad;
     const int zb0 = bz * zbk, zb1 = std::min(zb0 + zbk, nz);
-    for (int tid = 0; tid < NT; ++tid) {
+    for (int tid = 0; tid < nth; ++tid) {
       const int gx = x0 + tid % TXS, gy = y0 + tid / TXS;
       if (!(gx <= rx1 && gy <= ry1)) continue;  // inactive thread
       if (gx < 0 || gy < 0 || gx >= nx || gy >= ny) {
@@ -701,7 +743,8 @@ long long replay_gather_layout(int nx, int ny, int nz, const int* plo, const int
     }
   };
   if (!p.split) {
-    const int TXS = ab ? TileG::TXS : TileSq::TXS, TYS = ab ? TileG::TYS : TileSq::TYS;
+    const int TXS = p.small ? TileS::TXS : ab ? TileG::TXS : TileSq::TXS,
+              TYS = p.small ? TileS::TYS : ab ? TileG::TYS : TileSq::TYS;
     for (int bz = 0; bz < p.nzb; ++bz)
       for (int by = 0; by < p.TYT; ++by)
         for (int bx = 0; bx < p.TXT * nrhs; ++bx) {

@@ -101,6 +101,10 @@ void launch_block_gram(const BlockCols& X, const BlockCols& Y, double* partial, 
 template <class R>
 void launch_block_update(const BlockCols& X, cx<R>* Y, int q, const double* C, double beta, cudaStream_t s);
 void block_init_attrs();
+// Grids of at most this many nodes run as many small blocks (8 x 8 tiles, two
+// planes), in the gather form on every level, forward and adjoint: see k_fwd_small.
+constexpr long long kSmallNodes = 1LL << 17;
+
 namespace march {
 // forward stencil in single precision, every level (hz_march.cuh)
 // Small grids take the gather-form kernels of hz_fwd_gather.cu, on every level:

@@ -2250,7 +2250,12 @@ extern "C" hz_status iofd_residual_static(hz_handle* H, int level, int op, int p
     const bool adj0 = (op == HZ_OP_A_ADJ || op == HZ_OP_B_ADJ);
     // partial sums of the launch that will run (forward and adjoint tile differently)
     const LevelView<double> lvd = view<double>(H, level);
-    const long long need = resid_blocks(lv, level, nrhs, adj0, lvd.zblock, lvd.zblock_f) * nrhs;
+    // (very small grids run more, smaller blocks than their limit was set for: 32 x 8
+    // tiles of four planes)
+    const long long launch = resid_blocks(lv, level, nrhs, adj0, lvd.zblock, lvd.zblock_f);
+    const long long need = nrhs * (lv.N <= kSmallNodes
+                                       ? (long long)((lv.nx + 31) / 32) * ((lv.ny + 7) / 8) * ((lv.nz + 3) / 4)
+                                       : launch);
     HZ_REQUIRE(need <= kResidStaticPartials,
                "grid too large for the static scratch (" + std::to_string(need) + " block partial sums > " +
                    std::to_string(kResidStaticPartials) + ")");
@@ -2264,14 +2269,15 @@ extern "C" hz_status iofd_residual_static(hz_handle* H, int level, int op, int p
     HZ_CK(cudaMemsetAsync(red.count, 0, sizeof(unsigned) * nrhs, st));
     const bool adj = adj0;
     const bool shifted = (op == HZ_OP_B || op == HZ_OP_B_ADJ);
+    // a launch of more blocks than the limit was counted on leaves its norm to a
+    // pass of at most 608 blocks
+    const bool fused =
+        (adj || precision != HZ_C64 ? launch : fwd_blocks_c64(lv, nrhs)) * nrhs <= kResidStaticPartials;
     if (precision == HZ_C64) {
       StencilCall<float> c = call<float>(H, level, shifted, nrhs);
       c.x = (const cx<float>*)x;
       c.g = (const cx<float>*)g;
       c.y = (cx<float>*)r;
-      // the limit above is counted on the complex128 launch in either precision; a
-      // complex64 launch of more blocks leaves its norm to a pass of at most 608
-      const bool fused = adj || fwd_blocks_c64(lv, nrhs) * nrhs <= kResidStaticPartials;
       if (fused) c.red = red;
       launch_stencil<float>(c, M_RESID, OP_AB, adj, st);
       if (!fused) launch_norm2<float>(c.y, (int)lv.N, nrhs, red, st);
@@ -2280,8 +2286,9 @@ extern "C" hz_status iofd_residual_static(hz_handle* H, int level, int op, int p
       c.x = (const cx<double>*)x;
       c.g = (const cx<double>*)g;
       c.y = (cx<double>*)r;
-      c.red = red;
+      if (fused) c.red = red;
       launch_stencil<double>(c, M_RESID, OP_AB, adj, st);
+      if (!fused) launch_norm2<double>(c.y, (int)lv.N, nrhs, red, st);
     }
     HZ_LAUNCHED();
   });

@@ -33,8 +33,13 @@ extern template void fwd_init_attrs<double, M_J2>();
 extern template void fwd_init_attrs<double, M_JSWEEP>();
 extern template void fwd_init_attrs<double, M_AWIN>();
 
-constexpr int TX = 32, TY = 8, NT = TX * TY;
-constexpr int PW = TX + 2, PH = TY + 2, PLANE = PW * PH;
+// tiles of the adjoint kernel: 32 x 8 columns, 8 x 8 on very small grids
+template <int TX_, int TY_>
+struct ATile {
+  static constexpr int TX = TX_, TY = TY_, NT = TX_ * TY_, PW = TX_ + 2, PLANE = PW * (TY_ + 2);
+};
+using ATileL = ATile<32, 8>;
+using ATileS = ATile<8, 8>;
 
 // ----------------------------------------------------------------------------
 // adjoint kernel
@@ -56,22 +61,22 @@ constexpr int PW = TX + 2, PH = TY + 2, PLANE = PW * PH;
 // (27 complex coefficients per output node) is what it gains: bound by issue in
 // single precision and by the FP64 rate in double.
 constexpr int kAdjF = 7;  // fields in shared memory: u_0..u_3, v_0..v_2
-template <class R>
+template <class R, class AT>
 struct AdjSmem {
-  static constexpr size_t o_tab = (size_t)2 * kAdjF * PLANE * sizeof(cx<R>);
+  static constexpr size_t o_tab = (size_t)2 * kAdjF * AT::PLANE * sizeof(cx<R>);
   static size_t bytes(int opk, int ns) {
     return o_tab + sizeof(R) * (opk == OPK_Q ? (size_t)kCtQ : (size_t)(kCtCA + kCtK + kCtT)) * ns;
   }
 };
 
-template <class R, int MODE, int OPK, bool GEN>
+template <class R, int MODE, int OPK, bool GEN, class AT>
 __device__ __forceinline__ void adj_tile(const StencilCall<R>& a, unsigned char* smem, double* sRed, int zblock,
                                          int tiles_x) {
   constexpr bool Q = OPK == OPK_Q, B = OPK == OPK_B;
-  constexpr int NF = GEN ? kAdjF : 4;
+  constexpr int TX = AT::TX, TY = AT::TY, NT = AT::NT, PW = AT::PW, PLANE = AT::PLANE;
   const LevelView<R>& L = a.lv;
   cx<R>* sF = reinterpret_cast<cx<R>*>(smem);
-  R* sT = reinterpret_cast<R*>(smem + AdjSmem<R>::o_tab);
+  R* sT = reinterpret_cast<R*>(smem + AdjSmem<R, AT>::o_tab);
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
   const int ns = a.tab.nseg + 1;
   const R ds = a.tab.ds, inv_ds = a.tab.inv_ds;
@@ -249,12 +254,13 @@ __device__ __forceinline__ void adj_tile(const StencilCall<R>& a, unsigned char*
   }
 }
 
-template <class R, int MODE, int OPK>
-__global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 1) k_adj(StencilCall<R> a, int zblock, int tiles_x) {
+template <class R, int MODE, int OPK, class AT>
+__global__ void __launch_bounds__(AT::NT, (sizeof(R) == 4 ? 3 : 1) * (256 / AT::NT)) k_adj(StencilCall<R> a, int zblock, int tiles_x) {
+  constexpr int TX = AT::TX, TY = AT::TY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double sRed[32];
   if constexpr (OPK == OPK_Q) {
-    adj_tile<R, MODE, OPK, false>(a, smem_raw, sRed, zblock, tiles_x);
+    adj_tile<R, MODE, OPK, false, AT>(a, smem_raw, sRed, zblock, tiles_x);
   } else {
     // a source node in the PML of any axis, the halo's included?
     const LevelView<R>& L = a.lv;
@@ -262,8 +268,8 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 1) k_adj(StencilCall<
     const int zb0 = blockIdx.z * zblock, zb1 = min(zb0 + zblock, L.nz);
     const bool plain = x0 - 1 >= L.plain_lo[0] && x0 + TX <= L.plain_hi[0] && y0 - 1 >= L.plain_lo[1] &&
                        y0 + TY <= L.plain_hi[1] && zb0 - 1 >= L.plain_lo[2] && zb1 <= L.plain_hi[2];
-    if (plain) adj_tile<R, MODE, OPK, false>(a, smem_raw, sRed, zblock, tiles_x);
-    else adj_tile<R, MODE, OPK, true>(a, smem_raw, sRed, zblock, tiles_x);
+    if (plain) adj_tile<R, MODE, OPK, false, AT>(a, smem_raw, sRed, zblock, tiles_x);
+    else adj_tile<R, MODE, OPK, true, AT>(a, smem_raw, sRed, zblock, tiles_x);
   }
 }
 
@@ -293,23 +299,35 @@ __global__ void k_j1(StencilCall<R> a, int adjoint) {
 // ----------------------------------------------------------------------------
 // launchers
 // ----------------------------------------------------------------------------
-// z-block of the adjoint kernel (32 x 8 tiles over the whole grid)
-static int adj_zblock(int nx, int ny, int nz, int nrhs) {
-  const long long tiles = (long long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY) * nrhs;
-  const long long want = 152LL * 2 * 4;
-  const long long nzb = (want + tiles - 1) / tiles;
-  int zb = (int)((nz + nzb - 1) / nzb);
-  return std::min(std::max(zb, 4), kMaxZb);
+// tiling of the adjoint kernel over the whole grid (zblock > 0 forces it)
+struct AdjPlan {
+  int tw, th, zb, nx, ny, nz;  // tile, planes per block, blocks per axis
+};
+static AdjPlan adj_plan(int nx, int ny, int nz, int nrhs, int zblock = 0) {
+  AdjPlan p;
+  const bool small = (long long)nx * ny * nz <= kSmallNodes;
+  p.tw = small ? ATileS::TX : ATileL::TX;
+  p.th = small ? ATileS::TY : ATileL::TY;
+  p.nx = (nx + p.tw - 1) / p.tw;
+  p.ny = (ny + p.th - 1) / p.th;
+  const long long tiles = (long long)p.nx * p.ny * nrhs, want = 152LL * 2 * 4, nzb = (want + tiles - 1) / tiles;
+  p.zb = small ? kMinZblock : std::min(std::max((int)((nz + nzb - 1) / nzb), 4), kMaxZb);
+  if (zblock > 0) p.zb = zblock;
+  p.nz = (nz + p.zb - 1) / p.zb;
+  return p;
 }
 
+template <class R, int MODE, int OPK, class AT>
+static void launch_adj_at(const StencilCall<R>& c, const AdjPlan& p, cudaStream_t s) {
+  count_launch();
+  k_adj<R, MODE, OPK, AT><<<dim3(p.nx * c.nrhs, p.ny, p.nz), dim3(AT::TX, AT::TY),
+                            AdjSmem<R, AT>::bytes(OPK, c.tab.nseg + 1), s>>>(c, p.zb, p.nx);
+}
 template <class R, int MODE, int OPK>
 static void launch_adj_t(const StencilCall<R>& c, cudaStream_t s) {
-  const LevelView<R>& L = c.lv;
-  const int zb = adj_zblock(L.nx, L.ny, L.nz, c.nrhs);
-  const int tiles_x = (L.nx + TX - 1) / TX;
-  dim3 grid(tiles_x * c.nrhs, (L.ny + TY - 1) / TY, (L.nz + zb - 1) / zb);
-  count_launch();
-  k_adj<R, MODE, OPK><<<grid, dim3(TX, TY), AdjSmem<R>::bytes(OPK, c.tab.nseg + 1), s>>>(c, zb, tiles_x);
+  const AdjPlan p = adj_plan(c.lv.nx, c.lv.ny, c.lv.nz, c.nrhs);
+  if (p.tw == ATileS::TX) launch_adj_at<R, MODE, OPK, ATileS>(c, p, s);
+  else launch_adj_at<R, MODE, OPK, ATileL>(c, p, s);
 }
 
 // forward operator kind of a call: A (real shell coefficients) unless the mass
@@ -334,7 +352,7 @@ void launch_stencil(const StencilCall<R>& c, int mode, int op, bool adjoint, cud
     if constexpr (sizeof(R) == sizeof(float)) {
       if (mode == M_AWIN || march::takes(mode, c.lv.nx, c.lv.ny, c.lv.nz, c.nrhs)) march::launch(c, mode, opk, s);
       else gather::launch_fwd_gather(c, mode, op, s);
-    } else if (c.lv.level > 0) {
+    } else if (mode != M_AWIN && (c.lv.level > 0 || c.lv.N <= kSmallNodes)) {
       gather::launch_fwd_gather(c, mode, op, s);
     } else if (op == OP_Q) {
       launch_fwd<R, M_APPLY>(c, opk, s);
@@ -367,7 +385,8 @@ void launch_stencil(const StencilCall<R>& c, int mode, int op, bool adjoint, cud
 // size of the per-block partial-sum array its fused reductions need).
 long long stencil_blocks_per_rhs(int level, int nx, int ny, int nz, const int* plain_lo, const int* plain_hi,
                                  int nrhs, int zblock, int zblock_f) {
-  if (level > 0) return gather::gather_blocks_per_rhs(nx, ny, nz, plain_lo, plain_hi, nrhs, zblock, zblock_f);
+  if (level > 0 || (long long)nx * ny * nz <= kSmallNodes)
+    return gather::gather_blocks_per_rhs(nx, ny, nz, plain_lo, plain_hi, nrhs, zblock, zblock_f);
   const int zb = zblock > 0 ? zblock : choose_zblock(nx, ny, nz, nrhs);
   const FwdPlan p = plan_layout(nx, ny, nz, plain_lo, plain_hi, true, zb, zblock_f);
   return p.blocks();
@@ -376,8 +395,8 @@ long long stencil_blocks_per_rhs(int level, int nx, int ny, int nz, const int* p
 // Blocks per right-hand side of an adjoint stencil launch with nrhs
 // right-hand sides (zblock > 0: that z-block instead of the launch's own).
 long long adj_blocks_per_rhs(int nx, int ny, int nz, int nrhs, int zblock) {
-  const int zb = zblock > 0 ? zblock : adj_zblock(nx, ny, nz, nrhs);
-  return (long long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY) * ((nz + zb - 1) / zb);
+  const AdjPlan p = adj_plan(nx, ny, nz, nrhs, zblock);
+  return (long long)p.nx * p.ny * p.nz;
 }
 
 // Host replay of the forward launch layout and of the kernels' block and
@@ -393,9 +412,9 @@ long long replay_fwd_layout(int level, int nx, int ny, int nz, const int* plo, c
                             int zblock, int zblock_f, unsigned char* counts, long long* blocks) {
   // the single-precision launch has a layout of its own (march, small grids gather)
   long long single = march::replay_layout(nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f);
-  if (level == 0 && !march::takes(M_J2, nx, ny, nz, 1))
+  if (level == 0 && (long long)nx * ny * nz > kSmallNodes && !march::takes(M_J2, nx, ny, nz, 1))
     single += gather::replay_gather_layout(nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f, nullptr, nullptr);
-  if (level > 0)
+  if (level > 0 || (long long)nx * ny * nz <= kSmallNodes)
     return single + gather::replay_gather_layout(nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f, counts, blocks);
   const bool ab = op == OP_AB;
   const int zb = zblock > 0 ? zblock : choose_zblock(nx, ny, nz, nrhs);
@@ -473,17 +492,16 @@ long long replay_fwd_layout(int level, int nx, int ny, int nz, const int* plo, c
 // adj_zblock planes per block unless zblock > 0): per-node write counts of
 // right-hand side 0 (or null) and the blocks per right-hand side.
 long long replay_adj_layout(int nx, int ny, int nz, int nrhs, int zblock, unsigned char* counts, long long* blocks) {
-  const int zb = zblock > 0 ? zblock : adj_zblock(nx, ny, nz, nrhs);
-  const int tx = (nx + TX - 1) / TX, ty = (ny + TY - 1) / TY, tz = (nz + zb - 1) / zb;
-  if (blocks) *blocks = (long long)tx * ty * tz;
+  const AdjPlan p = adj_plan(nx, ny, nz, nrhs, zblock);
+  if (blocks) *blocks = (long long)p.nx * p.ny * p.nz;
   if (counts)
-    for (int bz = 0; bz < tz; ++bz)
-      for (int by = 0; by < ty; ++by)
-        for (int bx = 0; bx < tx; ++bx)
-          for (int t = 0; t < NT; ++t) {
-            const int gx = bx * TX + t % TX, gy = by * TY + t / TX;
+    for (int bz = 0; bz < p.nz; ++bz)
+      for (int by = 0; by < p.ny; ++by)
+        for (int bx = 0; bx < p.nx; ++bx)
+          for (int t = 0; t < p.tw * p.th; ++t) {
+            const int gx = bx * p.tw + t % p.tw, gy = by * p.th + t / p.tw;
             if (gx >= nx || gy >= ny) continue;
-            for (int z = bz * zb; z < std::min(bz * zb + zb, nz); ++z) {
+            for (int z = bz * p.zb; z < std::min(bz * p.zb + p.zb, nz); ++z) {
               unsigned char& c = counts[((size_t)z * ny + gy) * nx + gx];
               if (c < 255) ++c;
             }
@@ -493,8 +511,10 @@ long long replay_adj_layout(int nx, int ny, int nz, int nrhs, int zblock, unsign
 
 template <class R, int MODE, int OPK>
 static void set_adj_attr() {
-  cudaFuncSetAttribute(k_adj<R, MODE, OPK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)AdjSmem<R>::bytes(OPK, kMaxSeg + 1));
+  cudaFuncSetAttribute(k_adj<R, MODE, OPK, ATileL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)AdjSmem<R, ATileL>::bytes(OPK, kMaxSeg + 1));
+  cudaFuncSetAttribute(k_adj<R, MODE, OPK, ATileS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)AdjSmem<R, ATileS>::bytes(OPK, kMaxSeg + 1));
 }
 template <class R>
 static void set_adj_attrs() {
