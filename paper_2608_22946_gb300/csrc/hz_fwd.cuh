@@ -21,10 +21,10 @@
 // tiles, to the in-plane differences the corrections need) and added to the
 // three rows it touches: it completes the row below (as that row's "+1"
 // plane), adds to its own row, and opens the row above (as its "-1" plane).
-// Live state per column: two accumulators per right-hand side and the
-// coefficients of three rows.  The coefficients of a row are evaluated once,
-// from kappa, and serve every right-hand side the block carries (a block
-// processes RB right-hand sides of the same tile).
+// Live state per column: two accumulators and the coefficients of three rows,
+// each row's evaluated once, from kappa.  A block serves one right-hand side.
+// Runs complex128 (single precision: hz_march.cuh); its kernels are bound by the
+// FP64 rate.
 //
 // Coefficients: C_m(kappa) = (L_m(eta) - kappa^2 M_m(eta)) / ell^2 with the
 // stiffness and mass shell weights L_m, M_m of the cubic Hermite alpha's and
@@ -100,21 +100,16 @@ struct Shapes<2> {
 constexpr long long kCoarseNodes = 8LL << 20;
 constexpr long long kFusedNodes = 1LL << 20;
 
-// ring depth by precision, mode and right-hand sides per block; PREF = NSTG - 2
-// planes are in flight, and the stage of the previous plane stays readable
-template <class R, int MODE, int RB>
-struct FStages {
-  static constexpr int v = (sizeof(R) == 8 || MODE == M_J2 || RB > 1) ? 3 : 6;
-};
-
-template <class R, int MODE, int OPK, class TS, int RB>
+template <class R, int MODE, int OPK, class TS>
 struct FLayout {
-  static constexpr int NSTG = FStages<R, MODE, RB>::v;
+  // ring depth: PREF = NSTG - 2 planes are in flight, and the stage of the previous
+  // plane stays readable
+  static constexpr int NSTG = 3;
   static constexpr size_t CXB = sizeof(cx<R>);
   static constexpr size_t a16(size_t x) { return (x + 15) & ~(size_t)15; }
-  static constexpr size_t ring = (size_t)NSTG * RB * TS::PLN * CXB;
+  static constexpr size_t ring = (size_t)NSTG * TS::PLN * CXB;
   static constexpr size_t dring = MODE == M_J2 ? (size_t)NSTG * TS::PLN * CXB : 0;
-  static constexpr size_t y1 = MODE == M_J2 ? (size_t)RB * TS::PLN * CXB : 0;
+  static constexpr size_t y1 = MODE == M_J2 ? (size_t)TS::PLN * CXB : 0;
   static constexpr size_t kap = (size_t)NSTG * TS::NT * TS::NPX * sizeof(R);
   static constexpr int tabn = (OPK == OPK_Q ? kCtQ : kCtCA + (OPK == OPK_B ? kCtK : 0) + kCtT) * (kMaxSeg + 1);
   static constexpr size_t tab = (size_t)tabn * sizeof(R);
@@ -363,15 +358,15 @@ __device__ __forceinline__ cx<R> contrib(const CT& C, const RowT<R>& T, cx<R> c,
 
 // ----------------------------------------------------------------------------
 // one block: tile (x0, y0) of shape TS writing columns up to (rx1, ry1), z-block
-// blockIdx.z, right-hand sides rhs0 .. rhs0 + RB - 1
+// blockIdx.z, right-hand side rhs
 // ----------------------------------------------------------------------------
 // FORM: 0 shell (x and y outside the PML), 3 y stretched, 2 x and y stretched.
 // ZP: some row of the block lies in the z-PML (blocks wholly between the two
 // z-layers carry no z-correction code at all).
-template <class R, int MODE, int OPK, int FORM, bool ZP, class TS, int RB>
+template <class R, int MODE, int OPK, int FORM, bool ZP, class TS>
 __device__ __forceinline__ void fwd_tile(const StencilCall<R>& a, unsigned char* smem, int zblock, int x0, int y0,
-                                         int rx1, int ry1, int rhs0, unsigned bid, unsigned nblk) {
-  using LY = FLayout<R, MODE, OPK, TS, RB>;
+                                         int rx1, int ry1, int rhs, unsigned bid, unsigned nblk) {
+  using LY = FLayout<R, MODE, OPK, TS>;
   constexpr int NSTG = LY::NSTG, PREF = NSTG - 2;
   constexpr int NPX = TS::NPX, PWS = TS::PWS, PLN = TS::PLN, NT = TS::NT, NSLOT = TS::NSLOT;
   constexpr bool CPLX = OPK == OPK_B;
@@ -467,10 +462,9 @@ __device__ __forceinline__ void fwd_tile(const StencilCall<R>& a, unsigned char*
     const int q = zb0 - 1 + kk;
     const bool zin = (unsigned)q < (unsigned)nz;
     const int zo = zin ? q * plane_sz : 0;
-#pragma unroll
-    for (int r = 0; r < RB; ++r) {
-      const cx<R>* Xr = a.x + (size_t)(rhs0 + r) * (size_t)xs + (zin ? zo - (long long)xz0 * plane_sz : 0);
-      cx<R>* dst = sX + ((size_t)st * RB + r) * PLN + tid;
+    {
+      const cx<R>* Xr = a.x + (size_t)rhs * (size_t)xs + (zin ? zo - (long long)xz0 * plane_sz : 0);
+      cx<R>* dst = sX + (size_t)st * PLN + tid;
 #pragma unroll
       for (int j = 0; j < NSLOT; ++j)
         if (slot_ok(j)) fcp_async<sizeof(cx<R>)>(dst + j * NT, Xr + go[j], zin && gin[j]);
@@ -505,17 +499,13 @@ __device__ __forceinline__ void fwd_tile(const StencilCall<R>& a, unsigned char*
   // the rows' kappa and evaluate the weights where a z-correction needs them.
   constexpr bool HOLD_T = CORR;
   constexpr bool HOLD_K = !CORR && ZP;
-  cx<R> accP[RB][NPX], accM[RB][NPX];
+  cx<R> accP[NPX], accM[NPX];
   CT C[3][NPX];
   RowT<R> Th[HOLD_T ? 3 : 1][NPX];
   R kq[HOLD_K ? 3 : 1][NPX];
-  R nrm2[RB];
+  R nrm2 = 0;
 #pragma unroll
-  for (int r = 0; r < RB; ++r) {
-    nrm2[r] = 0;
-#pragma unroll
-    for (int i = 0; i < NPX; ++i) accP[r][i] = accM[r][i] = mkc<R>(0, 0);
-  }
+  for (int i = 0; i < NPX; ++i) accP[i] = accM[i] = mkc<R>(0, 0);
 #pragma unroll
   for (int sl = 0; sl < (HOLD_T ? 3 : 1); ++sl)
 #pragma unroll
@@ -536,20 +526,18 @@ __device__ __forceinline__ void fwd_tile(const StencilCall<R>& a, unsigned char*
     const bool o1 = k + 3 <= nplanes;      // row p+1 lies in this z-block
     const bool o0 = k >= 1 && k + 2 <= nplanes;
     const bool o3 = k >= 2;                // row p-1 completes
-    const cx<R>* Xs = sX + (size_t)st * RB * PLN;
-    const cx<R>* Xsp = sX + (size_t)stp * RB * PLN;
+    const cx<R>* Xs = sX + (size_t)st * PLN;
+    const cx<R>* Xsp = sX + (size_t)stp * PLN;
 
     // own-column values of row p-1 read early (their latency overlaps the step)
-    cx<R> gq[RB][NPX];
+    [[maybe_unused]] cx<R> gq[NPX];
     constexpr bool WANT_G = MODE == M_RESID || MODE == M_JSWEEP || MODE == M_J2;
     if constexpr (WANT_G) {
       const cx<R>* src = (MODE == M_J2) ? a.base : a.g;
       if (o3 && src) {
 #pragma unroll
-        for (int r = 0; r < RB; ++r)
-#pragma unroll
-          for (int i = 0; i < NPX; ++i)
-            gq[r][i] = act[i] ? src[(size_t)(rhs0 + r) * (size_t)N + (p - 1) * plane_sz + col0 + i] : mkc<R>(0, 0);
+        for (int i = 0; i < NPX; ++i)
+          gq[i] = act[i] ? src[(size_t)rhs * (size_t)N + (p - 1) * plane_sz + col0 + i] : mkc<R>(0, 0);
       }
     }
 
@@ -610,30 +598,19 @@ __device__ __forceinline__ void fwd_tile(const StencilCall<R>& a, unsigned char*
         if (!slot_ok(j)) continue;
         const int li = tid + j * NT;
         const cx<R> d = Ds[li];
-#pragma unroll
-        for (int r = 0; r < RB; ++r) sY1[(size_t)r * PLN + li] = om * (d * Xs[(size_t)r * PLN + li]);
+        sY1[li] = om * (d * Xs[li]);
       }
       __syncthreads();
     }
 
-#pragma unroll
-    for (int r = 0; r < RB; ++r) {
-      const cx<R>* P = (MODE == M_J2) ? sY1 + (size_t)r * PLN : Xs + (size_t)r * PLN;
+    {
+      const cx<R>* P = (MODE == M_J2) ? sY1 : Xs;
       cx<R> v[3][NPX + 2];
 #pragma unroll
       for (int row = 0; row < 3; ++row) {
         const cx<R>* q = P + (ty + row) * PWS + NPX * tx;
-        if constexpr (NPX == 2 && sizeof(R) == 4) {
-          const float4 u0 = *reinterpret_cast<const float4*>(q);
-          const float4 u1 = *reinterpret_cast<const float4*>(q + 2);
-          v[row][0] = mkc<R>(u0.x, u0.y);
-          v[row][1] = mkc<R>(u0.z, u0.w);
-          v[row][2] = mkc<R>(u1.x, u1.y);
-          v[row][3] = mkc<R>(u1.z, u1.w);
-        } else {
 #pragma unroll
-          for (int j = 0; j < NPX + 2; ++j) v[row][j] = q[j];
-        }
+        for (int j = 0; j < NPX + 2; ++j) v[row][j] = q[j];
       }
       cx<R> sv[NPX + 2];
 #pragma unroll
@@ -660,41 +637,39 @@ __device__ __forceinline__ void fwd_tile(const StencilCall<R>& a, unsigned char*
           cfma(Bc, exm_[i], Vm);
         }
         if (o3) {
-          const cx<R> h = accM[r][i] + contrib<+1, CORR, ZP>(C[CM][i], T3[i], c, e, kk, Ac, Bc, zq3, ez3);
+          const cx<R> h = accM[i] + contrib<+1, CORR, ZP>(C[CM][i], T3[i], c, e, kk, Ac, Bc, zq3, ez3);
           if (act[i]) {
             const int idx = (p - 1) * plane_sz + col0 + i;
             cx<R> out;
             if constexpr (MODE == M_APPLY || MODE == M_AWIN) {
               out = h;
             } else if constexpr (MODE == M_RESID) {
-              out = gq[r][i] - h;
-              nrm2[r] += abs2(out);
+              out = gq[i] - h;
+              nrm2 += abs2(out);
             } else if constexpr (MODE == M_J2) {
-              const cx<R> g0 = Xsp[(size_t)r * PLN + lc0 + i];
+              const cx<R> g0 = Xsp[lc0 + i];
               const cx<R> d0 = sD[(size_t)stp * PLN + lc0 + i];
               out = om * (d0 * g0) + om * (d0 * (g0 - h));
-              if (a.base) out += gq[r][i];
+              if (a.base) out += gq[i];
             } else {  // M_JSWEEP
-              const cx<R> x0c = Xsp[(size_t)r * PLN + lc0 + i];
+              const cx<R> x0c = Xsp[lc0 + i];
               const cx<R> d0 = a.dinv[idx];
-              out = x0c + om * (d0 * (gq[r][i] - h));
+              out = x0c + om * (d0 * (gq[i] - h));
             }
-            a.y[(size_t)(rhs0 + r) * (size_t)ys + idx - (long long)zr0 * plane_sz] = out;
+            a.y[(size_t)rhs * (size_t)ys + idx - (long long)zr0 * plane_sz] = out;
           }
         }
-        if (o0) accP[r][i] += contrib<0, CORR, ZP>(C[CP][i], T0[i], c, e, kk, Ac, Bc, zq0, ez0);
-        if (o1) accM[r][i] = contrib<-1, CORR, ZP>(C[CN][i], T1[i], c, e, kk, Ac, Bc, zq1, ez1);
+        if (o0) accP[i] += contrib<0, CORR, ZP>(C[CP][i], T0[i], c, e, kk, Ac, Bc, zq0, ez0);
+        if (o1) accM[i] = contrib<-1, CORR, ZP>(C[CN][i], T1[i], c, e, kk, Ac, Bc, zq1, ez1);
       }
     }
     // row p+1 (now in accM) is next step's role-0 row; row p becomes its row to complete
 #pragma unroll
-    for (int r = 0; r < RB; ++r)
-#pragma unroll
-      for (int i = 0; i < NPX; ++i) {
-        const cx<R> t = accP[r][i];
-        accP[r][i] = accM[r][i];
-        accM[r][i] = t;
-      }
+    for (int i = 0; i < NPX; ++i) {
+      const cx<R> t = accP[i];
+      accP[i] = accM[i];
+      accM[i] = t;
+    }
     stp = st;
     st = (st + 1 == NSTG) ? 0 : st + 1;
     sti = (sti + 1 == NSTG) ? 0 : sti + 1;
@@ -710,10 +685,9 @@ __device__ __forceinline__ void fwd_tile(const StencilCall<R>& a, unsigned char*
 
   if constexpr (MODE == M_RESID) {
     if (a.red.out) {
-#pragma unroll
-      for (int r = 0; r < RB; ++r) {
-        const unsigned rr = (unsigned)(rhs0 + r);
-        double s = block_sum((double)nrm2[r], sRed, tid, NT);
+      {
+        const unsigned rr = (unsigned)rhs;
+        double s = block_sum((double)nrm2, sRed, tid, NT);
         if (tid == 0) a.red.partial[(size_t)rr * nblk + bid] = s;
         if (last_block_arrive(a.red.count + rr, nblk, tid)) {
           double t = 0.0;
@@ -744,90 +718,82 @@ __device__ __forceinline__ bool block_in_zpml(const StencilCall<R>& a, int zbloc
 // ----------------------------------------------------------------------------
 // kernels
 // ----------------------------------------------------------------------------
-// resident blocks per SM the register allocation targets
-template <class R, int RB, int NT, int NPX, int OPK>
-struct FMinB {
-  static constexpr int v = sizeof(R) == 8 ? 1 : (NT == 256 ? (NPX == 1 && RB == 1 && OPK != OPK_B ? 3 : 2) : 4);
-};
-
 // the PML-free rectangle (shell rows)
-template <class R, int MODE, int OPK, int RB, int SS>
-__global__ void __launch_bounds__(Shapes<SS>::Rect::NT,
-                                  FMinB<R, RB, Shapes<SS>::Rect::NT, Shapes<SS>::Rect::NPX, OPK>::v)
+template <class R, int MODE, int OPK, int SS>
+__global__ void __launch_bounds__(Shapes<SS>::Rect::NT, 1)
     k_fwd_rect(StencilCall<R> a, int zblock, TileMap tm) {
   using ShRect = typename Shapes<SS>::Rect;
   extern __shared__ __align__(16) unsigned char fsm[];
-  const int ng = a.nrhs / RB;
+  const int ng = a.nrhs;
   const int g = blockIdx.x % ng, t = blockIdx.x / ng;
   const unsigned bid = (unsigned)(tm.bid_offset + t + tm.ntx * (blockIdx.y + gridDim.y * blockIdx.z));
   const int x0 = tm.ox + t * ShRect::TWN, y0 = tm.oy + (int)blockIdx.y * ShRect::TYT;
   const unsigned nb = (unsigned)tm.nblk_total;
   if (block_in_zpml<MODE>(a, zblock))
-    fwd_tile<R, MODE, OPK, 0, true, ShRect, RB>(a, fsm, zblock, x0, y0, tm.rx1, tm.ry1, g * RB, bid, nb);
+    fwd_tile<R, MODE, OPK, 0, true, ShRect>(a, fsm, zblock, x0, y0, tm.rx1, tm.ry1, g, bid, nb);
   else
-    fwd_tile<R, MODE, OPK, 0, false, ShRect, RB>(a, fsm, zblock, x0, y0, tm.rx1, tm.ry1, g * RB, bid, nb);
+    fwd_tile<R, MODE, OPK, 0, false, ShRect>(a, fsm, zblock, x0, y0, tm.rx1, tm.ry1, g, bid, nb);
 }
 
 // the PML frame around it: strips below and above the rectangle (y stretched)
 // and left and right of it (x stretched, y too in the corners)
-template <class R, int MODE, int OPK, int RB, int SS>
-__global__ void __launch_bounds__(Shapes<SS>::Wide::NT, FMinB<R, RB, Shapes<SS>::Wide::NT, 2, OPK>::v)
+template <class R, int MODE, int OPK, int SS>
+__global__ void __launch_bounds__(Shapes<SS>::Wide::NT, 1)
     k_fwd_frame(StencilCall<R> a, int zblock, TileMap tm) {
   using ShWide = typename Shapes<SS>::Wide;
   using ShTall = typename Shapes<SS>::Tall;
   static_assert(ShWide::NT == ShTall::NT, "one block size for both frame tile shapes");
   extern __shared__ __align__(16) unsigned char fsm[];
-  const int ng = a.nrhs / RB;
+  const int ng = a.nrhs;
   const int g = blockIdx.x % ng, t = blockIdx.x / ng;
   const FrameTile f = decode_frame(tm, t);
   const unsigned bid = (unsigned)(tm.bid_offset + t + tm.count * blockIdx.z);
   const unsigned nb = (unsigned)tm.nblk_total;
   const bool zp = block_in_zpml<MODE>(a, zblock);
   if (f.wide) {
-    if (zp) fwd_tile<R, MODE, OPK, 3, true, ShWide, RB>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g * RB, bid, nb);
-    else fwd_tile<R, MODE, OPK, 3, false, ShWide, RB>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g * RB, bid, nb);
+    if (zp) fwd_tile<R, MODE, OPK, 3, true, ShWide>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g, bid, nb);
+    else fwd_tile<R, MODE, OPK, 3, false, ShWide>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g, bid, nb);
   } else {
-    if (zp) fwd_tile<R, MODE, OPK, 2, true, ShTall, RB>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g * RB, bid, nb);
-    else fwd_tile<R, MODE, OPK, 2, false, ShTall, RB>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g * RB, bid, nb);
+    if (zp) fwd_tile<R, MODE, OPK, 2, true, ShTall>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g, bid, nb);
+    else fwd_tile<R, MODE, OPK, 2, false, ShTall>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g, bid, nb);
   }
 }
 
 // a whole (small) grid in one launch, the row form chosen per tile; Q_h (shell
 // form everywhere) always takes this path
-template <class R, int MODE, int OPK, int RB, int SS>
-__global__ void __launch_bounds__(Shapes<SS>::Rect::NT, sizeof(R) == 8 ? 1 : 2) k_fwd_grid(StencilCall<R> a, int zblock,
-                                                                                           TileMap tm) {
+template <class R, int MODE, int OPK, int SS>
+__global__ void __launch_bounds__(Shapes<SS>::Rect::NT, 1) k_fwd_grid(StencilCall<R> a, int zblock, TileMap tm) {
   using ShRect = typename Shapes<SS>::Rect;
   extern __shared__ __align__(16) unsigned char fsm[];
-  const int ng = a.nrhs / RB;
+  const int ng = a.nrhs;
   const int g = blockIdx.x % ng, t = blockIdx.x / ng;
   const unsigned bid = (unsigned)(t + tm.ntx * (blockIdx.y + gridDim.y * blockIdx.z));
   const int x0 = t * ShRect::TWN, y0 = (int)blockIdx.y * ShRect::TYT;
   const int rx1 = a.lv.nx - 1, ry1 = a.lv.ny - 1;
   const unsigned nb = (unsigned)tm.nblk_total;
   if constexpr (OPK == OPK_Q) {
-    fwd_tile<R, MODE, OPK, 0, false, ShRect, RB>(a, fsm, zblock, x0, y0, rx1, ry1, g * RB, bid, nb);
+    fwd_tile<R, MODE, OPK, 0, false, ShRect>(a, fsm, zblock, x0, y0, rx1, ry1, g, bid, nb);
   } else {
     const bool zp = block_in_zpml<MODE>(a, zblock);
     if (grid_tile_form(x0, y0, ShRect::TWN, ShRect::TYT, a.lv.nx, a.lv.ny, a.lv.plain_lo, a.lv.plain_hi) == 0) {
-      if (zp) fwd_tile<R, MODE, OPK, 0, true, ShRect, RB>(a, fsm, zblock, x0, y0, rx1, ry1, g * RB, bid, nb);
-      else fwd_tile<R, MODE, OPK, 0, false, ShRect, RB>(a, fsm, zblock, x0, y0, rx1, ry1, g * RB, bid, nb);
+      if (zp) fwd_tile<R, MODE, OPK, 0, true, ShRect>(a, fsm, zblock, x0, y0, rx1, ry1, g, bid, nb);
+      else fwd_tile<R, MODE, OPK, 0, false, ShRect>(a, fsm, zblock, x0, y0, rx1, ry1, g, bid, nb);
     } else {
-      fwd_tile<R, MODE, OPK, 2, true, ShRect, RB>(a, fsm, zblock, x0, y0, rx1, ry1, g * RB, bid, nb);
+      fwd_tile<R, MODE, OPK, 2, true, ShRect>(a, fsm, zblock, x0, y0, rx1, ry1, g, bid, nb);
     }
   }
 }
 
 // rectangle and frame tiles of a small grid in one launch (tile set 2): block t
 // < RW * RH (tm.ntx * tm.rows) is a rectangle tile, the rest frame tiles
-template <class R, int MODE, int OPK, int RB>
-__global__ void __launch_bounds__(256, sizeof(R) == 8 ? 1 : 2) k_fwd_fused(StencilCall<R> a, int zblock, TileMap tm) {
+template <class R, int MODE, int OPK>
+__global__ void __launch_bounds__(256, 1) k_fwd_fused(StencilCall<R> a, int zblock, TileMap tm) {
   using SRect = Shapes<2>::Rect;
   using SWide = Shapes<2>::Wide;
   using STall = Shapes<2>::Tall;
   static_assert(SRect::NT == 256 && SWide::NT == 256 && STall::NT == 256, "one block size");
   extern __shared__ __align__(16) unsigned char fsm[];
-  const int ng = a.nrhs / RB;
+  const int ng = a.nrhs;
   const int g = blockIdx.x % ng, t = blockIdx.x / ng;
   const int nrect = tm.ntx * tm.nrow;
   const unsigned bid = (unsigned)(t + (nrect + tm.count) * blockIdx.z);
@@ -835,32 +801,32 @@ __global__ void __launch_bounds__(256, sizeof(R) == 8 ? 1 : 2) k_fwd_fused(Stenc
   const bool zp = block_in_zpml<MODE>(a, zblock);
   if (t < nrect) {
     const int x0 = tm.px0 + (t % tm.ntx) * SRect::TWN, y0 = tm.py0 + (t / tm.ntx) * SRect::TYT;
-    if (zp) fwd_tile<R, MODE, OPK, 0, true, SRect, RB>(a, fsm, zblock, x0, y0, tm.px1, tm.py1, g * RB, bid, nb);
-    else fwd_tile<R, MODE, OPK, 0, false, SRect, RB>(a, fsm, zblock, x0, y0, tm.px1, tm.py1, g * RB, bid, nb);
+    if (zp) fwd_tile<R, MODE, OPK, 0, true, SRect>(a, fsm, zblock, x0, y0, tm.px1, tm.py1, g, bid, nb);
+    else fwd_tile<R, MODE, OPK, 0, false, SRect>(a, fsm, zblock, x0, y0, tm.px1, tm.py1, g, bid, nb);
     return;
   }
   const FrameTile f = decode_frame(tm, t - nrect);
   if (f.wide) {
-    if (zp) fwd_tile<R, MODE, OPK, 3, true, SWide, RB>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g * RB, bid, nb);
-    else fwd_tile<R, MODE, OPK, 3, false, SWide, RB>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g * RB, bid, nb);
+    if (zp) fwd_tile<R, MODE, OPK, 3, true, SWide>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g, bid, nb);
+    else fwd_tile<R, MODE, OPK, 3, false, SWide>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g, bid, nb);
   } else {
-    fwd_tile<R, MODE, OPK, 2, true, STall, RB>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g * RB, bid, nb);
+    fwd_tile<R, MODE, OPK, 2, true, STall>(a, fsm, zblock, f.x0, f.y0, f.rx1, f.ry1, g, bid, nb);
   }
 }
 
-template <class R, int MODE, int OPK, int RB>
+template <class R, int MODE, int OPK>
 constexpr size_t fwd_smem_fused() {
-  return std::max(std::max(FLayout<R, MODE, OPK, Shapes<2>::Rect, RB>::bytes,
-                           FLayout<R, MODE, OPK, Shapes<2>::Wide, RB>::bytes),
-                  FLayout<R, MODE, OPK, Shapes<2>::Tall, RB>::bytes);
+  return std::max(std::max(FLayout<R, MODE, OPK, Shapes<2>::Rect>::bytes,
+                           FLayout<R, MODE, OPK, Shapes<2>::Wide>::bytes),
+                  FLayout<R, MODE, OPK, Shapes<2>::Tall>::bytes);
 }
 
-template <class R, int MODE, int OPK, int RB, int SS>
-constexpr size_t fwd_smem_rect() { return FLayout<R, MODE, OPK, typename Shapes<SS>::Rect, RB>::bytes; }
-template <class R, int MODE, int OPK, int RB, int SS>
+template <class R, int MODE, int OPK, int SS>
+constexpr size_t fwd_smem_rect() { return FLayout<R, MODE, OPK, typename Shapes<SS>::Rect>::bytes; }
+template <class R, int MODE, int OPK, int SS>
 constexpr size_t fwd_smem_frame() {
-  return std::max(FLayout<R, MODE, OPK, typename Shapes<SS>::Wide, RB>::bytes,
-                  FLayout<R, MODE, OPK, typename Shapes<SS>::Tall, RB>::bytes);
+  return std::max(FLayout<R, MODE, OPK, typename Shapes<SS>::Wide>::bytes,
+                  FLayout<R, MODE, OPK, typename Shapes<SS>::Tall>::bytes);
 }
 
 }  // namespace hz

@@ -1,4 +1,6 @@
-// Gather-form forward stencil of the coarse levels (2h, 4h) for sm_103a.
+// Gather-form forward stencil for sm_103a: complex128 on the coarse levels (2h, 4h),
+// complex64 on grids too small for the march (march::takes), both on very small grids
+// of any level (kSmallNodes).
 //
 // Operator as in hz_fwd.cuh (Sec. 2.2, Eq. iofd-shell-form / Eq.
 // pml-second-difference).  Design for small, L2-resident grids, where latency

@@ -113,45 +113,45 @@ inline FwdPlan plan_fwd_mode(StencilCall<R> c, bool ab) {
   return plan_fwd(c, ab);
 }
 
-template <class R, int MODE, int OPK, int RB, int SS>
+template <class R, int MODE, int OPK, int SS>
 void launch_fwd_split(const StencilCall<R>& c, const FwdPlan& p, int ng, int nblk_total, cudaStream_t s);
 
-template <class R, int MODE, int OPK, int RB, int SS>
+template <class R, int MODE, int OPK, int SS>
 void launch_fwd_ss(const StencilCall<R>& c, const FwdPlan& p, cudaStream_t s) {
-  const int ng = c.nrhs / RB;
+  const int ng = c.nrhs;
   const int nblk_total = (int)p.blocks();
   if (OPK == OPK_Q || !p.split) {
     TileMap tm = p.frame;
     tm.ntx = p.GW;
     tm.nblk_total = nblk_total;
     count_launch();
-    k_fwd_grid<R, MODE, OPK, RB, SS><<<dim3(p.GW * ng, p.GH, p.nzb), Shapes<SS>::Rect::NT,
-                                       fwd_smem_rect<R, MODE, OPK, RB, SS>(), s>>>(c, p.zb, tm);
+    k_fwd_grid<R, MODE, OPK, SS><<<dim3(p.GW * ng, p.GH, p.nzb), Shapes<SS>::Rect::NT,
+                                       fwd_smem_rect<R, MODE, OPK, SS>(), s>>>(c, p.zb, tm);
     return;
   }
-  if constexpr (OPK != OPK_Q) launch_fwd_split<R, MODE, OPK, RB, SS>(c, p, ng, nblk_total, s);
+  if constexpr (OPK != OPK_Q) launch_fwd_split<R, MODE, OPK, SS>(c, p, ng, nblk_total, s);
 }
 
-template <class R, int MODE, int OPK, int RB>
-void launch_fwd_rb(const StencilCall<R>& c, cudaStream_t s) {
+template <class R, int MODE, int OPK>
+void launch_fwd_opk(const StencilCall<R>& c, cudaStream_t s) {
   const FwdPlan p = plan_fwd_mode<R, MODE>(c, OPK != OPK_Q);
   if constexpr (OPK != OPK_Q) {
     if (p.fused) {
       TileMap tm = p.frame;
       tm.nblk_total = (int)p.blocks();
-      const int ng = c.nrhs / RB;
+      const int ng = c.nrhs;
       count_launch();
-      k_fwd_fused<R, MODE, OPK, RB><<<dim3((p.RW * p.RH + tm.count) * ng, 1, p.nzb), 256,
-                                      fwd_smem_fused<R, MODE, OPK, RB>(), s>>>(c, p.zb, tm);
+      k_fwd_fused<R, MODE, OPK><<<dim3((p.RW * p.RH + tm.count) * ng, 1, p.nzb), 256,
+                                      fwd_smem_fused<R, MODE, OPK>(), s>>>(c, p.zb, tm);
       return;
     }
   }
-  if (p.ss == 0) launch_fwd_ss<R, MODE, OPK, RB, 0>(c, p, s);
-  else launch_fwd_ss<R, MODE, OPK, RB, 1>(c, p, s);
+  if (p.ss == 0) launch_fwd_ss<R, MODE, OPK, 0>(c, p, s);
+  else launch_fwd_ss<R, MODE, OPK, 1>(c, p, s);
 }
 
 // the rectangle and frame launches of a split application
-template <class R, int MODE, int OPK, int RB, int SS>
+template <class R, int MODE, int OPK, int SS>
 void launch_fwd_split(const StencilCall<R>& c, const FwdPlan& p, int ng, int nblk_total, cudaStream_t s) {
   TileMap ti = p.frame;
   ti.ox = p.frame.px0;
@@ -173,12 +173,12 @@ void launch_fwd_split(const StencilCall<R>& c, const FwdPlan& p, int ng, int nbl
     cudaStreamWaitEvent(s2, c.fork, 0);
   }
   count_launch();
-  k_fwd_rect<R, MODE, OPK, RB, SS><<<dim3(p.RW * ng, p.RH, p.nzb), Shapes<SS>::Rect::NT,
-                                     fwd_smem_rect<R, MODE, OPK, RB, SS>(), s>>>(c, p.zb, ti);
+  k_fwd_rect<R, MODE, OPK, SS><<<dim3(p.RW * ng, p.RH, p.nzb), Shapes<SS>::Rect::NT,
+                                     fwd_smem_rect<R, MODE, OPK, SS>(), s>>>(c, p.zb, ti);
   if (tp.count > 0) {
     count_launch();
-    k_fwd_frame<R, MODE, OPK, RB, SS><<<dim3(tp.count * ng, 1, p.nzbf), Shapes<SS>::Wide::NT,
-                                        fwd_smem_frame<R, MODE, OPK, RB, SS>(), s2>>>(c, p.zbf, tp);
+    k_fwd_frame<R, MODE, OPK, SS><<<dim3(tp.count * ng, 1, p.nzbf), Shapes<SS>::Wide::NT,
+                                        fwd_smem_frame<R, MODE, OPK, SS>(), s2>>>(c, p.zbf, tp);
   }
   if (fork) {
     cudaEventRecord(c.join, s2);
@@ -186,50 +186,24 @@ void launch_fwd_split(const StencilCall<R>& c, const FwdPlan& p, int ng, int nbl
   }
 }
 
-// right-hand sides per block: two for complex64 (the coefficients of three
-// rows and two accumulators per right-hand side stay in registers), one for
-// complex128 (its kernels are bound by the FP64 rate)
-template <class R, int MODE>
-constexpr int fwd_rb_max() {
-  return sizeof(R) == 8 ? 1 : 2;
-}
-inline int fwd_pick_rb(int nrhs, int rbmax) { return (rbmax >= 2 && nrhs % 2 == 0) ? 2 : 1; }
-
-template <class R, int MODE, int OPK>
-void launch_fwd_opk(const StencilCall<R>& c, cudaStream_t s) {
-  constexpr int RBM = fwd_rb_max<R, MODE>();
-  if constexpr (RBM >= 2) {
-    if (fwd_pick_rb(c.nrhs, RBM) == 2) {
-      launch_fwd_rb<R, MODE, OPK, 2>(c, s);
-      return;
-    }
-  }
-  launch_fwd_rb<R, MODE, OPK, 1>(c, s);
-}
-
-template <class R, int MODE, int OPK, int RB, int SS>
+template <class R, int MODE, int OPK, int SS>
 void fwd_attrs_ss() {
-  cudaFuncSetAttribute(k_fwd_grid<R, MODE, OPK, RB, SS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)fwd_smem_rect<R, MODE, OPK, RB, SS>());
+  cudaFuncSetAttribute(k_fwd_grid<R, MODE, OPK, SS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)fwd_smem_rect<R, MODE, OPK, SS>());
   if constexpr (OPK != OPK_Q) {
-    cudaFuncSetAttribute(k_fwd_rect<R, MODE, OPK, RB, SS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)fwd_smem_rect<R, MODE, OPK, RB, SS>());
-    cudaFuncSetAttribute(k_fwd_frame<R, MODE, OPK, RB, SS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)fwd_smem_frame<R, MODE, OPK, RB, SS>());
+    cudaFuncSetAttribute(k_fwd_rect<R, MODE, OPK, SS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)fwd_smem_rect<R, MODE, OPK, SS>());
+    cudaFuncSetAttribute(k_fwd_frame<R, MODE, OPK, SS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)fwd_smem_frame<R, MODE, OPK, SS>());
   }
-}
-template <class R, int MODE, int OPK, int RB>
-void fwd_attrs_rb() {
-  fwd_attrs_ss<R, MODE, OPK, RB, 0>();
-  fwd_attrs_ss<R, MODE, OPK, RB, 1>();
-  if constexpr (OPK != OPK_Q)
-    cudaFuncSetAttribute(k_fwd_fused<R, MODE, OPK, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)fwd_smem_fused<R, MODE, OPK, RB>());
 }
 template <class R, int MODE, int OPK>
 void fwd_attrs_opk() {
-  fwd_attrs_rb<R, MODE, OPK, 1>();
-  if constexpr (fwd_rb_max<R, MODE>() >= 2) fwd_attrs_rb<R, MODE, OPK, 2>();
+  fwd_attrs_ss<R, MODE, OPK, 0>();
+  fwd_attrs_ss<R, MODE, OPK, 1>();
+  if constexpr (OPK != OPK_Q)
+    cudaFuncSetAttribute(k_fwd_fused<R, MODE, OPK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)fwd_smem_fused<R, MODE, OPK>());
 }
 
 // Entry points of one (precision, mode): instantiated in hz_fwd.cu, one

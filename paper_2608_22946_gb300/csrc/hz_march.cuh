@@ -20,7 +20,7 @@
 //    two-float adds (re, im);
 //  - the gather form keeps (c, e, k) of one plane and what the plane before adds to
 //    the next row, so a row's weights are needed in one place, its completion;
-//  - the weights of A are cubics on quarter segments (16 multiply-adds fewer loads
+//  - the weights of A are cubics on parts of a segment (16 multiply-adds fewer loads
 //    and steps than the quintics on whole ones); kappa's segment comes from a
 //    round-to-nearest add instead of conversions, and the local coordinate is
 //    measured in segments so that one subtraction gives it;

@@ -488,7 +488,7 @@ long long replay_fwd_layout(int level, int nx, int ny, int nz, const int* plo, c
   return bad;
 }
 
-// Host replay of the adjoint launch layout (32 x 8 tiles over the whole grid,
+// Host replay of the adjoint launch layout (tiles of adj_plan over the whole grid,
 // adj_zblock planes per block unless zblock > 0): per-node write counts of
 // right-hand side 0 (or null) and the blocks per right-hand side.
 long long replay_adj_layout(int nx, int ny, int nz, int nrhs, int zblock, unsigned char* counts, long long* blocks) {
