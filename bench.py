@@ -411,14 +411,14 @@ def run_gpu(args):
             result["stencil_batched_over_single"] = (N * nrhs / t_k) / (N / t_1)
         result["roofline"] = {"bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
                               "frac": achieved / pk["hbm_gbs"], "traffic": traffic,
-                              "kernel": "k_fwd_rect + k_fwd_frame (A_h, complex64, fine grid, one application)",
+                              "kernel": "k_march (A_h, complex64, fine grid, one application)",
                               "peak_kind": pk_kind, "gupdates_per_s": N * nrhs / t_k / 1e9,
                               "avg_launch_ms": 1000 * t_k, "bytes_per_node": 20}
         t_j = time_apply(s, hz, 0, None, nrhs, stream, mode="jacobi")
         ach_j = 28 * N * nrhs / t_j / 1e9
         result["roofline_smoother"] = {"bound": "hbm", "achieved": ach_j, "peak": pk["hbm_gbs"], "unit": "GB/s",
                                        "frac": ach_j / pk["hbm_gbs"], "traffic": None,
-                                       "kernel": "k_fwd_rect + k_fwd_frame, two-sweep Jacobi map J_2(A_h) "
+                                       "kernel": "k_march, two-sweep Jacobi map J_2(A_h) "
                                                  "(complex64, fine grid)",
                                        "peak_kind": pk_kind, "gupdates_per_s": N * nrhs / t_j / 1e9,
                                        "avg_launch_ms": 1000 * t_j, "bytes_per_node": 28}
