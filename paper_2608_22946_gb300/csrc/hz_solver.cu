@@ -407,12 +407,14 @@ double poly_at(const Poly& p, double u) {
 }
 // power basis (in x = nsub u - b) of the cubic through p at the Chebyshev nodes of part b
 std::array<double, 4> part_cubic(const Poly& p, int nsub, int b) {
-  double x[4], f[4];
+  static const std::array<double, 4> x = [] {
+    std::array<double, 4> t;
+    for (int i = 0; i < 4; ++i) t[i] = 0.5 - 0.5 * std::cos(M_PI * (2 * i + 1) / 8.0);
+    return t;
+  }();
+  double f[4];
   std::array<double, 4> c{};
-  for (int i = 0; i < 4; ++i) {
-    x[i] = 0.5 - 0.5 * std::cos(M_PI * (2 * i + 1) / 8.0);
-    f[i] = poly_at(p, (b + x[i]) / nsub);
-  }
+  for (int i = 0; i < 4; ++i) f[i] = poly_at(p, (b + x[i]) / nsub);
   for (int s = 1; s < 4; ++s)  // Newton's divided differences, then the power basis
     for (int i = 3; i >= s; --i) f[i] = (f[i] - f[i - 1]) / (x[i] - x[i - s]);
   c[0] = f[3];
@@ -957,7 +959,7 @@ size_t red_partial_size(const Level* lev, int nrhs) {
     m = std::max(m, (size_t)std::max(f, a));
     for (int r = 1; r <= 2; ++r)  // (one and two right-hand sides per block tile differently)
       m = std::max(m, (size_t)march::blocks_per_rhs(lev[L].nx, lev[L].ny, lev[L].nz, lev[L].plain_lo, lev[L].plain_hi,
-                                                    r, kMinZblock, kMinZblock));
+                                                    r, kMinZblock, kMinZblock, lev[L].strip));
   }
   return m * nrhs;
 }
@@ -983,8 +985,10 @@ void plan_all(hz_handle* H, bool count_only) {
       }
     }
     lv.ctab_d = al.get<double>((size_t)kCtPerSeg * (kMaxSeg + 1));
-    lv.ctab_f = al.get<float>((size_t)kCtPerSeg * (kMaxSeg + 1));
-    lv.mtab_f = al.get<float>((size_t)march::mt_size(kMaxSeg + 1));
+    // one allocation and one copy for the two single-precision tables
+    static_assert(kCtPerSeg % 4 == 0, "the second table starts on a 16-byte boundary");
+    lv.ctab_f = al.get<float>((size_t)kCtPerSeg * (kMaxSeg + 1) + march::mt_size(kMaxSeg + 1));
+    if (lv.ctab_f) lv.mtab_f = lv.ctab_f + (size_t)kCtPerSeg * (kMaxSeg + 1);
   }
   H->lev[0].dinv_f[0] = al.get<cx<float>>(H->lev[0].N + 1);
   H->lev[1].dinv_f[1] = al.get<cx<float>>(H->lev[1].N + 1);
@@ -993,8 +997,8 @@ void plan_all(hz_handle* H, bool count_only) {
   H->tab_f = al.get<float>((size_t)kMaxSeg * kNumFn * 4);
   const int nr = H->max_nrhs;
   H->red_partial = al.get<double>(red_partial_size(H->lev, nr));
-  H->red_count = al.get<unsigned>(nr);
-  H->bot_err = al.get<int>(1);
+  H->red_count = al.get<unsigned>(nr + 1);  // the last one: the kernels' error flag
+  if (H->red_count) H->bot_err = reinterpret_cast<int*>(H->red_count + nr);
   H->cgs_skip = al.get<int>(nr);
   H->s_nrm = al.get<double>(nr);
   H->s_root = al.get<double>(nr);
@@ -1754,8 +1758,7 @@ hz_status hz_create(const hz_grid* grid, const double* c_dev, const hz_params* p
     HZ_LAUNCHED();
     auto t0 = std::chrono::steady_clock::now();
     plan_all(H, false);
-    HZ_CK(cudaMemsetAsync(H->red_count, 0, sizeof(unsigned) * max_nrhs, H->st));
-    HZ_CK(cudaMemsetAsync(H->bot_err, 0, sizeof(int), H->st));
+    HZ_CK(cudaMemsetAsync(H->red_count, 0, sizeof(unsigned) * (max_nrhs + 1), H->st));
     {
       // opt-in: on the 289^3 benchmark the ten grid barriers cost more than the
       // launch gaps they replace (15.0 against 14.2-14.5 ms per preconditioner call)
@@ -1813,12 +1816,12 @@ hz_status hz_create(const hz_grid* grid, const double* c_dev, const hz_params* p
         std::vector<double> ct_d, ct_s;
         build_coef_tables(coef, table_host, table_rows, ds, lv.ell, false, ct_d);
         build_coef_tables(coef, table_host, table_rows, ds, lv.ell, true, ct_s);
-        std::vector<float> ct_f(ct_s.begin(), ct_s.end());
+        std::vector<float> ct_f(ct_s.begin(), ct_s.end()), mt;
+        build_march_tables(coef, table_host, table_rows, ds, lv.ell, H->nsub, mt);
+        ct_f.resize((size_t)(lv.mtab_f - lv.ctab_f), 0.f);
+        ct_f.insert(ct_f.end(), mt.begin(), mt.end());
         HZ_CK(cudaMemcpy(lv.ctab_d, ct_d.data(), ct_d.size() * sizeof(double), cudaMemcpyHostToDevice));
         HZ_CK(cudaMemcpy(lv.ctab_f, ct_f.data(), ct_f.size() * sizeof(float), cudaMemcpyHostToDevice));
-        std::vector<float> mt;
-        build_march_tables(coef, table_host, table_rows, ds, lv.ell, H->nsub, mt);
-        HZ_CK(cudaMemcpy(lv.mtab_f, mt.data(), mt.size() * sizeof(float), cudaMemcpyHostToDevice));
       }
       launch_setup_kappa<double>(c_dev, H->g.nx + 1, H->g.ny + 1, H->g.nz + 1, H->g.n_pml, f, H->g.omega, lv.ell,
                                  lv.kap_d, H->st);
