@@ -581,7 +581,6 @@ __device__ __forceinline__ void tile_body(const StencilCall<float>& a, unsigned 
 // alternates with y and z, and the march alternates two instances of its step.
 constexpr int kCoreW = 64;                    // columns of a tile
 constexpr unsigned kRowB = 544;               // bytes of a row in shared memory: 68 values
-constexpr int kWaitLimit = 1 << 22;           // polls, 64 ns apart, before a wait gives up
 
 template <int MODE, int NPY, int RB>
 struct CoreSmem {
@@ -614,13 +613,14 @@ __device__ __forceinline__ bool mbar_try(unsigned b, unsigned ph) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait.  Once one has given up the thread waits no more: the kernel ends
-// with invalid results and the host reports it.
-__device__ __forceinline__ void mbar_wait(unsigned b, unsigned ph, bool& dead, int* err) {
+// Bounded wait (polls: 64 ns apart).  Once one has given up the thread waits no
+// more (dead, the planes asked for by then): the kernel ends with invalid results
+// and the host reports it.
+__device__ __forceinline__ void mbar_wait(unsigned b, unsigned ph, int& dead, int armed, int* err, unsigned polls) {
   if (dead) return;
   for (int i = 0; i < 16; ++i)
     if (mbar_try(b, ph)) return;  // (suspends for a while by itself)
-  for (int i = 0; i < kWaitLimit; ++i) {
+  for (unsigned i = 0; i < polls; ++i) {
     unsigned ok;
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
@@ -630,7 +630,7 @@ __device__ __forceinline__ void mbar_wait(unsigned b, unsigned ph, bool& dead, i
     if (ok) return;
     __nanosleep(64);
   }
-  dead = true;
+  dead = armed;
   if (err) atomicExch(err, 1);
 }
 template <int BYTES>
@@ -738,7 +738,7 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
   if (tid == 0) {
 #pragma unroll
     for (int i = 0; i < NSTG; ++i) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full + 8 * i) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full + 8 * i), "r"(1 + a.extra) : "memory");
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(empty + 8 * i), "r"(NT / 32) : "memory");
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -748,7 +748,9 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
   // Copies of plane k (thread 0).  Global row of the tile's first halo row in
   // plane 0 of right-hand side rhs0; rows of the same parity start at line
   // (row / 2), element (row & 1) nx + x0 - 1 of it.
-  bool dead = false;
+  // Once a wait of this thread has given up it copies no more: a copy that is only
+  // late must not have its stage armed and written a second time.
+  int dead = 0;
   const int row0 = (int)(rhs0 * mp.rows) + (zb0 - 1 - a.xz0) * L.ny + y0 - 1;
   const int rowd = (zb0 - 1) * L.ny + y0 - 1;
   auto fetch = [&](int k, int st) {
@@ -863,7 +865,7 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
   int st = 0;
   unsigned ph = 0;
   if constexpr (J2) {
-    mbar_wait(full, 0, dead, a.err);
+    mbar_wait(full, 0, dead, min(PREF, nplanes), a.err, a.polls);
     transform(0, 0);
   }
 
@@ -877,19 +879,20 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
     else fcp_commit();
     if constexpr (J2) {
       __syncthreads();  // plane k is transformed, every warp has left plane k - 1
-      if (tid == 0 && k + PREF < nplanes) fetch(k + PREF, s2);
+      if (tid == 0 && k + PREF < nplanes && !dead) fetch(k + PREF, s2);
       const int sn = st + 1 == NSTG ? 0 : st + 1;
       if (k + 1 < nplanes) {
-        mbar_wait(full + 8 * sn, ph ^ (sn == 0), dead, a.err);
+        mbar_wait(full + 8 * sn, ph ^ (sn == 0), dead, min(k + PREF + 1, nplanes), a.err, a.polls);
         transform(k + 1, sn);
       }
     } else {
       if (tid == 0 && k + PREF < nplanes) {
-        if (k + PREF >= NSTG) mbar_wait(empty + 8 * s2, (unsigned)((k + PREF) / NSTG - 1) & 1, dead, a.err);
-        fetch(k + PREF, s2);
+        if (k + PREF >= NSTG)
+          mbar_wait(empty + 8 * s2, (unsigned)((k + PREF) / NSTG - 1) & 1, dead, k + PREF, a.err, a.polls);
+        if (!dead) fetch(k + PREF, s2);
       }
       __syncwarp();
-      mbar_wait(full + 8 * st, ph, dead, a.err);
+      mbar_wait(full + 8 * st, ph, dead, min(k + PREF + 1, nplanes), a.err, a.polls);
     }
     // what the Jacobi map is added to (a ring for it would cost a block per SM)
     [[maybe_unused]] float2 bq[RB][NPY][2];
@@ -1009,11 +1012,13 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
     if (k + 1 < nplanes) step(std::integral_constant<int, 1>{}, k + 1);
   }
   fcp_wait<0>();
-  if (dead) {  // a wait gave up: let the copies in flight land (bounded) before the block ends
-    bool again = false;
-    for (int i = 0; i < NSTG; ++i) {
-      mbar_wait(full + 8 * i, 0, again, a.err);
-      mbar_wait(full + 8 * i, 1, again, a.err);
+  // A wait of the copying thread gave up: its copies in flight land (bounded, each
+  // stage on its own) before the block ends.  A stage's last copy completes the
+  // phase of its last plane; a thread that waited for every plane has none left.
+  if (tid == 0 && dead) {
+    for (int i = 0; i < min(NSTG, dead); ++i) {
+      int gone = 0;
+      mbar_wait(full + 8 * i, (unsigned)((dead - 1 - i) / NSTG) & 1, gone, 1, a.err, a.polls);
     }
   }
   if constexpr (MODE == M_RESID) reduce_norm<RB>(a, reinterpret_cast<double*>(smem + SM::o_red), nrm2, rhs0, bid, nblk);

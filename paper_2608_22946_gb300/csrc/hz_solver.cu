@@ -176,6 +176,7 @@ struct hz_handle {
   double* bot_partial_f = nullptr;
   double* bot_partial_d = nullptr;
   unsigned bot_spins = 1u << 23, bot_extra = 0;
+  unsigned copy_polls = 1u << 22, copy_extra = 0;  // waits of the single-precision march
 };
 
 namespace {
@@ -563,6 +564,8 @@ StencilCall<R> call(hz_handle* H, int L, bool shifted, int nrhs) {
   c.fork = H->ev_fork;
   c.join = H->ev_join;
   c.err = H->bot_err;
+  c.polls = H->copy_polls;
+  c.extra = H->copy_extra;
   return c;
 }
 
@@ -1768,6 +1771,11 @@ hz_status hz_create(const hz_grid* grid, const double* c_dev, const hz_params* p
       if (bt && bt[0] == '1') {
         H->bot_extra = 1;
         H->bot_spins = 4096;
+      }
+      const char* ct = std::getenv("HZ_COPY_TEST");  // makes every copy wait of the march run out (tests)
+      if (ct && ct[0] == '1') {
+        H->copy_extra = 1;
+        H->copy_polls = 4096;
       }
       if (H->coop_bottom) {
         H->bot_bar = H->al.get<unsigned>(2);
