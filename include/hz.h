@@ -50,10 +50,11 @@ typedef enum {
                          bottom-solve kernel (opt-in: environment HZ_PERSISTENT=1 when the
                          handle is created; all its blocks are co-resident by a cooperative
                          launch) did not release, within about a second.  The
-                         kernel finishes without waiting, its results are invalid, and the
-                         next helmholtz_solve or helmholtz_adjoint_grad on the handle
-                         returns this status (threegrid_precond, being asynchronous, does
-                         not read it).  The context stays usable. */
+                         kernel finishes without waiting and its results are invalid.
+                         helmholtz_solve and helmholtz_adjoint_grad return this status for
+                         their own launches.  iofd_apply, iofd_apply_window, iofd_jacobi,
+                         iofd_residual_static and threegrid_precond, being asynchronous, do
+                         not: hz_check tells.  The context stays usable. */
   HZ_ENONFINITE = 6   /* a NaN/Inf appeared in a residual norm */
 } hz_status;
 
@@ -242,6 +243,13 @@ hz_status iofd_jacobi(hz_handle* h, int level, int op, int precision, int nsweep
  * any stream capture.  Every call shares the one array: calls that overlap on
  * the GPU (concurrent streams, several handles) race and must be serialised. */
 hz_status iofd_residual_static(hz_handle* h, int level, int op, int precision, const void* g_dev, const void* x_dev,
+/* Did a bounded wait give up in an asynchronous call (see HZ_ETIMEOUT) since the
+ * last hz_check?  Waits for the work on `stream`, returns HZ_ETIMEOUT if so and
+ * HZ_OK if not, and forgets it.  A call whose wait gave up before a later
+ * helmholtz_solve or helmholtz_adjoint_grad on the handle is still reported here.
+ * Work on other streams must have been waited for by the caller. */
+hz_status hz_check(hz_handle* h, void* stream);
+
                                void* r_dev, double* norm2_dev, int nrhs, void* stream);
 
 /* z = M_h^{-1} r: one application of the three-grid preconditioner of

@@ -25,7 +25,7 @@ _STATUS = {0: "HZ_OK", 1: "HZ_EINVAL", 2: "HZ_ENOMEM", 3: "HZ_ECUDA", 4: "HZ_ENO
 EXPORTED = ["hz_default_params", "hz_create", "hz_destroy", "hz_last_error", "hz_workspace_bytes",
             "hz_set_params", "iofd_coeffs", "iofd_apply", "threegrid_precond", "helmholtz_solve",
             "helmholtz_adjoint_grad", "hz_kernel_launches", "iofd_residual_static", "hz_layout_check",
-            "iofd_jacobi", "iofd_apply_window"]
+            "iofd_jacobi", "iofd_apply_window", "hz_check"]
 
 
 class HzGrid(ctypes.Structure):
@@ -95,6 +95,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
                                          ctypes.c_int, vp]
     lib.hz_layout_check.argtypes = [P(HzGrid), ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                     ctypes.c_int, vp, P(ctypes.c_longlong), P(ctypes.c_longlong)]
+    lib.hz_check.argtypes = [vp, vp]
     lib.threegrid_precond.argtypes = [vp, vp, vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, vp]
     lib.helmholtz_solve.argtypes = [vp, P(HzSource), ctypes.c_int, vp, vp, P(HzStats)]
     lib.helmholtz_adjoint_grad.argtypes = [vp, P(HzSource), ctypes.c_int, P(ctypes.c_int), ctypes.c_int,
@@ -284,6 +285,12 @@ class Solver:
                                                 x.data_ptr(), r.data_ptr(),
                                                 n2.data_ptr(), nrhs, _stream_ptr(stream)))
         return r, n2
+
+    # -- hz_check ------------------------------------------------------------
+    def check(self, stream=None):
+        """Wait for the stream's work and raise HzError (HZ_ETIMEOUT) if a bounded
+        wait gave up in an asynchronous call since the last check."""
+        self._ok(self._lib.hz_check(self._h, _stream_ptr(stream)))
 
     # -- threegrid_precond ---------------------------------------------------
     def threegrid_precond(self, r, adjoint=False, out=None, stream=None):

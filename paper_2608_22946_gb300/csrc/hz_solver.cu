@@ -177,6 +177,7 @@ struct hz_handle {
   double* bot_partial_d = nullptr;
   unsigned bot_spins = 1u << 23, bot_extra = 0;
   unsigned copy_polls = 1u << 22, copy_extra = 0;  // waits of the single-precision march
+  bool earlier_err = false;  // a wait of an asynchronous call gave up (set_aside_wait_err)
 };
 
 namespace {
@@ -1587,17 +1588,34 @@ SolveOut solve_c128(hz_handle* H, const cx<double>* b, cx<double>* x, int nrhs, 
 }
 
 // A bounded wait that gave up (a copy of the forward stencil, a grid barrier of
-// the persistent bottom solve) sets a device flag (the kernel then finishes without waiting, its results
-// invalid); the synchronous entry points read and clear it.
-void check_bottom_err(hz_handle* H) {
-  if (!H->bot_err) return;
+// the persistent bottom solve) sets a device flag (the kernel then finishes
+// without waiting, its results invalid).  Reads and clears it, after the work on st.
+bool take_wait_err(hz_handle* H, cudaStream_t st) {
+  if (!H->bot_err) return false;
   int e = 0;
-  HZ_CK(cudaMemcpyAsync(&e, H->bot_err, sizeof(int), cudaMemcpyDeviceToHost, H->st));
-  HZ_CK(cudaStreamSynchronize(H->st));
+  HZ_CK(cudaMemcpyAsync(&e, H->bot_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  HZ_CK(cudaStreamSynchronize(st));
   if (e) {
-    HZ_CK(cudaMemsetAsync(H->bot_err, 0, sizeof(int), H->st));
-    HZ_CK(cudaStreamSynchronize(H->st));
-    throw Fail{HZ_ETIMEOUT, "a bounded wait of a kernel gave up; the results are invalid"};
+    HZ_CK(cudaMemsetAsync(H->bot_err, 0, sizeof(int), st));
+    HZ_CK(cudaStreamSynchronize(st));
+  }
+  return e != 0;
+}
+constexpr const char* kWaitErr = "a bounded wait of a kernel gave up; the results are invalid";
+// The synchronous entry points report the launches of their own call: a flag that an
+// earlier, asynchronous call left is put aside for hz_check.
+void set_aside_wait_err(hz_handle* H) {
+  if (take_wait_err(H, H->st)) H->earlier_err = true;
+}
+void check_bottom_err(hz_handle* H) {
+  if (take_wait_err(H, H->st)) throw Fail{HZ_ETIMEOUT, kWaitErr};
+}
+SolveOut solve_checked(hz_handle* H, const cx<double>* b, cx<double>* x, int nrhs, bool adj) {
+  try {
+    return solve_c128(H, b, x, nrhs, adj);
+  } catch (const Fail& f) {
+    if (f.st == HZ_ENONFINITE) check_bottom_err(H);  // a wait that gave up explains the NaN
+    throw;
   }
 }
 
@@ -2019,6 +2037,15 @@ hz_status iofd_jacobi(hz_handle* H, int level, int op, int precision, int nsweep
     H->st = old;
   });
 }
+hz_status hz_check(hz_handle* H, void* stream) {
+  if (!H) return HZ_EINVAL;
+  return run_guarded(H, [&] {
+    const bool now = take_wait_err(H, (cudaStream_t)stream), earlier = H->earlier_err;
+    H->earlier_err = false;
+    if (now || earlier) throw Fail{HZ_ETIMEOUT, kWaitErr};
+  });
+}
+
 
 hz_status threegrid_precond(hz_handle* H, const void* r, void* z, int nrhs, int adjoint, int precision, void* stream) {
   if (!H) return HZ_EINVAL;
@@ -2050,6 +2077,7 @@ hz_status helmholtz_solve(hz_handle* H, const hz_source* src, int nsrc, void* v_
   hz_status st = run_guarded(H, [&] {
     HZ_REQUIRE(src && v_dev && nsrc >= 1, "null argument or nsrc < 1");
     H->st = H->own;
+    set_aside_wait_err(H);
     HZ_CK(cudaDeviceSynchronize());  // inputs written on other streams are complete
     auto t0 = std::chrono::steady_clock::now();
     const long long N = H->lev[0].N;
@@ -2058,13 +2086,7 @@ hz_status helmholtz_solve(hz_handle* H, const hz_source* src, int nsrc, void* v_
       const int ns = std::min(H->max_nrhs, nsrc - s0);
       source_rhs(H, src + s0, ns, H->b128);  // b = Q_h f (Eq. iofd-complete-system)
       cx<double>* v = (cx<double>*)v_dev + (size_t)s0 * N;
-      SolveOut o;
-      try {
-        o = solve_c128(H, H->b128, v, ns, false);
-      } catch (const Fail& f) {
-        if (f.st == HZ_ENONFINITE) check_bottom_err(H);  // a barrier that gave up explains the NaN
-        throw;
-      }
+      const SolveOut o = solve_checked(H, H->b128, v, ns, false);
       tot.pc += o.pc;
       tot.passes += o.passes;
       tot.rel = std::max(tot.rel, o.rel);
@@ -2111,6 +2133,7 @@ hz_status helmholtz_adjoint_grad(hz_handle* H, const hz_source* src, int nsrc, c
   hz_status st = run_guarded(H, [&] {
     HZ_REQUIRE(src && rec && dobs && misfit && grad_dev && nsrc >= 1 && nrec >= 1, "null argument or empty set");
     H->st = H->own;
+    set_aside_wait_err(H);
     HZ_CK(cudaDeviceSynchronize());
     auto t0 = std::chrono::steady_clock::now();
     const Level& L0 = H->lev[0];
@@ -2147,7 +2170,7 @@ hz_status helmholtz_adjoint_grad(hz_handle* H, const hz_source* src, int nsrc, c
       const int ns = std::min(nr, nsrc - s0);
       upload_sources(H, src + s0, ns);
       q_apply<double>(H, false, H->f128, H->b128, ns);
-      SolveOut o = solve_c128(H, H->b128, H->vg, ns, false);
+      SolveOut o = solve_checked(H, H->b128, H->vg, ns, false);
       tot.pc += o.pc;
       tot.passes += o.passes;
       tot.rel = std::max(tot.rel, o.rel);
@@ -2170,7 +2193,7 @@ hz_status helmholtz_adjoint_grad(hz_handle* H, const hz_source* src, int nsrc, c
       launch_scatter<double>(H->recv, H->rec_dev, nrec, (int)N, ns, H->rf, H->st);  // R^T (R u - d)
       q_apply<double>(H, true, H->rf, H->b128, ns);                                 // Q^H R^T (R u - d)
       HZ_LAUNCHED();
-      SolveOut oa = solve_c128(H, H->b128, H->lg, ns, true);                         // A^H lambda = ...
+      SolveOut oa = solve_checked(H, H->b128, H->lg, ns, true);                      // A^H lambda = ...
       tot.pc += oa.pc;
       tot.passes += oa.passes;
       tot.rel = std::max(tot.rel, oa.rel);

@@ -51,3 +51,28 @@ def test_march_waits_give_up_and_are_reported(hz, monkeypatch, nrhs):
     y, ref = t.iofd_apply(x), t.iofd_apply(x.to(torch.complex128))
     assert float(torch.linalg.vector_norm(y.to(torch.complex128) - ref) / torch.linalg.vector_norm(ref)) <= 2e-6
     t.close()
+
+
+def test_earlier_give_up_is_not_reported_by_a_correct_solve(hz, monkeypatch):
+    """49^3: the window apply is a march whose waits run out, a solve runs no march.
+    The solve is right and returns so; hz_check reports the window apply, once."""
+    w = W.gaussian_lens(n=48, n_pml=8)
+    monkeypatch.setenv("HZ_COPY_TEST", "1")
+    s = hz.Solver(w.n, w.n_pml, w.h, w.omega, w.c, params=hz.default_params(tol=1e-6))
+    monkeypatch.delenv("HZ_COPY_TEST")
+    x = torch.zeros((1, 51) + s.level_shape[0][1:], dtype=torch.complex64, device="cuda")
+    s.check()
+    for check_first in (True, False):
+        s.iofd_apply_window(x, 0, 49)
+        if check_first:
+            with pytest.raises(hz.HzError) as e:
+                s.check()
+            assert e.value.status == hz.HZ_ETIMEOUT
+        _, _, st = s.helmholtz_solve(w.sources, want_u=False)
+        assert st["rel_res"] <= 1e-6
+        if not check_first:
+            with pytest.raises(hz.HzError) as e:
+                s.check()
+            assert e.value.status == hz.HZ_ETIMEOUT
+        s.check()
+    s.close()
