@@ -243,14 +243,14 @@ hz_status iofd_jacobi(hz_handle* h, int level, int op, int precision, int nsweep
  * any stream capture.  Every call shares the one array: calls that overlap on
  * the GPU (concurrent streams, several handles) race and must be serialised. */
 hz_status iofd_residual_static(hz_handle* h, int level, int op, int precision, const void* g_dev, const void* x_dev,
+                               void* r_dev, double* norm2_dev, int nrhs, void* stream);
+
 /* Did a bounded wait give up in an asynchronous call (see HZ_ETIMEOUT) since the
  * last hz_check?  Waits for the work on `stream`, returns HZ_ETIMEOUT if so and
  * HZ_OK if not, and forgets it.  A call whose wait gave up before a later
  * helmholtz_solve or helmholtz_adjoint_grad on the handle is still reported here.
  * Work on other streams must have been waited for by the caller. */
 hz_status hz_check(hz_handle* h, void* stream);
-
-                               void* r_dev, double* norm2_dev, int nrhs, void* stream);
 
 /* z = M_h^{-1} r: one application of the three-grid preconditioner of
  * Algorithm 1 (pre-smooth S_h(r;0), restrict r - A_h z_pre, K_2h, prolong and

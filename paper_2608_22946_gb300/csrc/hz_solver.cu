@@ -2037,6 +2037,7 @@ hz_status iofd_jacobi(hz_handle* H, int level, int op, int precision, int nsweep
     H->st = old;
   });
 }
+
 hz_status hz_check(hz_handle* H, void* stream) {
   if (!H) return HZ_EINVAL;
   return run_guarded(H, [&] {
@@ -2045,7 +2046,6 @@ hz_status hz_check(hz_handle* H, void* stream) {
     if (now || earlier) throw Fail{HZ_ETIMEOUT, kWaitErr};
   });
 }
-
 
 hz_status threegrid_precond(hz_handle* H, const void* r, void* z, int nrhs, int adjoint, int precision, void* stream) {
   if (!H) return HZ_EINVAL;
@@ -2077,8 +2077,8 @@ hz_status helmholtz_solve(hz_handle* H, const hz_source* src, int nsrc, void* v_
   hz_status st = run_guarded(H, [&] {
     HZ_REQUIRE(src && v_dev && nsrc >= 1, "null argument or nsrc < 1");
     H->st = H->own;
-    set_aside_wait_err(H);
     HZ_CK(cudaDeviceSynchronize());  // inputs written on other streams are complete
+    set_aside_wait_err(H);
     auto t0 = std::chrono::steady_clock::now();
     const long long N = H->lev[0].N;
     SolveOut tot;
@@ -2133,8 +2133,8 @@ hz_status helmholtz_adjoint_grad(hz_handle* H, const hz_source* src, int nsrc, c
   hz_status st = run_guarded(H, [&] {
     HZ_REQUIRE(src && rec && dobs && misfit && grad_dev && nsrc >= 1 && nrec >= 1, "null argument or empty set");
     H->st = H->own;
-    set_aside_wait_err(H);
     HZ_CK(cudaDeviceSynchronize());
+    set_aside_wait_err(H);
     auto t0 = std::chrono::steady_clock::now();
     const Level& L0 = H->lev[0];
     const long long N = L0.N;
