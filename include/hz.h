@@ -235,10 +235,8 @@ hz_status iofd_jacobi(hz_handle* h, int level, int op, int precision, int nsweep
  *   g_dev, x_dev   DEVICE inputs, r_dev DEVICE output (N_L * nrhs, `precision`);
  *                  r must not alias g or x.
  *   norm2_dev      DEVICE double, nrhs values out.
- * Limits: nrhs <= 64 and (blocks per rhs of the launch that runs -- forward
- * or adjoint, which tile differently; hz_layout_check reports both, and the
- * complex128 launch counts for either precision) * nrhs
- * <= 65536; larger problems return HZ_EINVAL with a message.  The first call on a device looks
+ * Limit: nrhs <= 64 (HZ_EINVAL beyond).  A launch of more blocks than there are
+ * partial sums leaves its norm to a second pass over r.  The first call on a device looks
  * up the array's device address (cudaGetSymbolAddress) and should come before
  * any stream capture.  Every call shares the one array: calls that overlap on
  * the GPU (concurrent streams, several handles) race and must be serialised. */

@@ -940,7 +940,8 @@ void level_dims(const hz_grid& g, int L, Level& lv) {
 
 // Block partial sums of one fused stencil reduction (forward or adjoint
 // launch) on level lv with nrhs right-hand sides, at the z-blocks it will run.
-// (The forward count is that of the complex128 launch; fwd_blocks_c64 has the complex64 one.)
+// (The forward count is that of the complex128 launch; fwd_blocks_c64 has the complex64
+// residual's.)
 long long resid_blocks(const Level& lv, int level, int nrhs, bool adjoint, int zblock, int zblock_f) {
   return adjoint ? adj_blocks_per_rhs(lv.nx, lv.ny, lv.nz, nrhs)
                  : stencil_blocks_per_rhs(level, lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nrhs, zblock, zblock_f);
@@ -2281,18 +2282,17 @@ extern "C" hz_status iofd_residual_static(hz_handle* H, int level, int op, int p
     HZ_REQUIRE(nrhs >= 1 && nrhs <= H->max_nrhs, "nrhs out of range");
     HZ_REQUIRE(nrhs <= kResidStaticMaxRhs, "nrhs exceeds the static scratch limit of 64 right-hand sides");
     const Level& lv = H->lev[level];
-    const bool adj0 = (op == HZ_OP_A_ADJ || op == HZ_OP_B_ADJ);
-    // partial sums of the launch that will run (forward and adjoint tile differently)
+    const bool adj = (op == HZ_OP_A_ADJ || op == HZ_OP_B_ADJ);
+    const bool shifted = (op == HZ_OP_B || op == HZ_OP_B_ADJ);
+    // Partial sums of the launch that runs (forward and adjoint, complex64 and
+    // complex128 tile differently).  Where they do not fit, the norm is a pass of its
+    // own over r, of at most 608 blocks per right-hand side, which always fits.
     const LevelView<double> lvd = view<double>(H, level);
-    // (very small grids run more, smaller blocks than their limit was set for: 32 x 8
-    // tiles of four planes)
-    const long long launch = resid_blocks(lv, level, nrhs, adj0, lvd.zblock, lvd.zblock_f);
-    const long long need = nrhs * (lv.N <= kSmallNodes
-                                       ? (long long)((lv.nx + 31) / 32) * ((lv.ny + 7) / 8) * ((lv.nz + 3) / 4)
-                                       : launch);
-    HZ_REQUIRE(need <= kResidStaticPartials,
-               "grid too large for the static scratch (" + std::to_string(need) + " block partial sums > " +
-                   std::to_string(kResidStaticPartials) + ")");
+    const long long blocks = !adj && precision == HZ_C64
+                                 ? fwd_blocks_c64(lv, nrhs)
+                                 : resid_blocks(lv, level, nrhs, adj, lvd.zblock, lvd.zblock_f);
+    const bool fused = blocks * nrhs <= kResidStaticPartials;
+    static_assert(608 * kResidStaticMaxRhs <= kResidStaticPartials, "the norm pass fits");
     double* base = resid_static_scratch();
     cudaStream_t st = (cudaStream_t)stream;
     Reduce red;
@@ -2301,12 +2301,6 @@ extern "C" hz_status iofd_residual_static(hz_handle* H, int level, int op, int p
     red.count = reinterpret_cast<unsigned*>(base + kResidStaticPartials);
     // the arrival counters must start at zero (the last block also resets them)
     HZ_CK(cudaMemsetAsync(red.count, 0, sizeof(unsigned) * nrhs, st));
-    const bool adj = adj0;
-    const bool shifted = (op == HZ_OP_B || op == HZ_OP_B_ADJ);
-    // a launch of more blocks than the limit was counted on leaves its norm to a
-    // pass of at most 608 blocks
-    const bool fused =
-        (adj || precision != HZ_C64 ? launch : fwd_blocks_c64(lv, nrhs)) * nrhs <= kResidStaticPartials;
     if (precision == HZ_C64) {
       StencilCall<float> c = call<float>(H, level, shifted, nrhs);
       c.x = (const cx<float>*)x;
