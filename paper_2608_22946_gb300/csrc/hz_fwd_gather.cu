@@ -19,6 +19,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "hz_fwd.cuh"
 #include "hz_gram_solve.cuh"
 #include "hz_kernels.h"
 
@@ -125,6 +126,16 @@ __device__ __forceinline__ cx<R> stiff_mass(const Part<R, false>& m, const Part<
               qb * ((R)2 * ((m.k + p.k) - (m.e + p.e)));
   Mv = a1 * o.c + w1 * (o.e + m.c + p.c) + w2 * (o.k + m.e + p.e) + w3 * (m.k + p.k);
   return S12 + abz * S3 + acz * D3;
+}
+
+// The z terms alone: cz (T(+1) + T(-1) - 2 T(0)) + dz (T(+1) - T(-1)).
+template <class R>
+__device__ __forceinline__ cx<R> stiff_z(const Part<R, false>& m, const Part<R, false>& o, const Part<R, false>& p,
+                                         const RowT<R>& t, cx<R> cz, cx<R> dz) {
+  const cx<R> T3m = t.qb * m.k + t.q5 * m.e + t.a4 * m.c;
+  const cx<R> T30 = t.qb * o.k + t.q5 * o.e + t.a4 * o.c;
+  const cx<R> T3p = t.qb * p.k + t.q5 * p.e + t.a4 * p.c;
+  return dz * (T3p - T3m) + cz * ((T3p + T3m) - (R)2 * T30);
 }
 
 // General row (PML tiles).  With sb = (abar_x + abar_y)/2 and db = (abar_x - abar_y)/2,
@@ -237,7 +248,11 @@ __host__ __device__ __forceinline__ FrameTile decode_frame(const TileMap& m, int
 // Row forms: 0 shell (x and y outside the PML), 1 PML along x only, 2 general,
 // 3 PML along y only.  Forms 1 and 3 drop the first-difference term of the
 // PML-free axis, whose achk is exactly zero.
-template <class R, int MODE, int OP, int FORM, class TL>
+// CW (single precision, fine level): the shell weights C = (L - kappa^2 M) / ell^2 and,
+// for B, K = kappa^2 M / ell^2 come combined, as the level's quintics (hz_fwd.cuh), and
+// PML rows add their corrections to the shell row.  Forming L - kappa^2 M per row
+// rounds both: 49^3 homogeneous, A, 1.07e-7 of the norm against 5.4e-8.
+template <class R, int MODE, int OP, int FORM, class TL, bool CW = false>
 __device__ __forceinline__ void fwd_body(const StencilCall<R>& a, int zblock, int bz, const TileMap& tm, int rhs, int x0,
                                          int y0, int rx1, int ry1, unsigned bid, cx<R>* sX, cx<R>* sD, cx<R>* sY1,
                                          const R* sTab, double* sRed, R (*sKc)[TL::NTH], cx<R> (*sGc)[TL::NTH]) {
@@ -267,10 +282,18 @@ __device__ __forceinline__ void fwd_body(const StencilCall<R>& a, int zblock, in
   cx<R> abx = mkc<R>(1, 0), acx = mkc<R>(0, 0), aby = mkc<R>(1, 0), acy = mkc<R>(0, 0);
   if (GEN && OP == OP_AB) {
     int cxi = min(gx, L.nx - 1), cyi = min(gy, L.ny - 1);
-    abx = L.abar[0][cxi];
-    acx = L.achk[0][cxi];
-    aby = L.abar[1][cyi];
-    acy = L.achk[1][cyi];
+    if constexpr (CW) {  // (abar - 1) and achk, times -1 / ell^2
+      const cx<R> xp = L.eps[0][0][cxi], xm = L.eps[0][1][cxi], yp = L.eps[1][0][cyi], ym = L.eps[1][1][cyi];
+      abx = (R)0.5 * (xp + xm);
+      acx = (R)0.5 * (xp - xm);
+      aby = (R)0.5 * (yp + ym);
+      acy = (R)0.5 * (yp - ym);
+    } else {
+      abx = L.abar[0][cxi];
+      acx = L.achk[0][cxi];
+      aby = L.abar[1][cyi];
+      acy = L.achk[1][cyi];
+    }
   }
   const cx<R> sbxy = (R)0.5 * (abx + aby), dbxy = (R)0.5 * (abx - aby);
 
@@ -393,6 +416,45 @@ __device__ __forceinline__ void fwd_body(const StencilCall<R>& a, int zblock, in
         table_eval<R, 5, 3>(sTab, nseg, ds, inv_ds, eta_star(kap_prev), bv);
         if constexpr (!GEN) out = q_row(wm, w0, wp, bv);
         else out = mkc<R>(0, 0);
+      } else if constexpr (CW) {
+        const int ns = nseg + 1;
+        R u, wc[4];
+        const int seg = seg_exact(kap_prev, ns, ds, inv_ds, u);
+        horner_pm<R, 4, 5>(sTab + seg * kCtCA, u, wc);
+        const cx<R> N1 = w0.e + (wm.c + wp.c);
+        const cx<R> N2 = w0.k + (wm.e + wp.e);
+        const cx<R> N3 = wm.k + wp.k;
+        cx<R> Hx = mkc<R>(0, 0);
+        if (GEN || z < zpl_lo || z > zpl_hi) {
+          const RowT<R> t = eval_t(sTab + ct_off_T(ns), seg, u);
+          const R av[5] = {0, 0, 0, t.a4, (R)4 * t.q5};
+          const cx<R> zp = L.eps[2][0][z], zm = L.eps[2][1][z];
+          cx<R> Mv;
+          if constexpr (GEN)
+            Hx = stiff_mass<FORM>(wm, w0, wp, av, sbxy, dbxy, acx, acy, (R)0.5 * (zp + zm), (R)0.5 * (zp - zm), Mv);
+          else
+            Hx = stiff_z(wm, w0, wp, t, (R)0.5 * (zp + zm), (R)0.5 * (zp - zm));
+        }
+        Hx += wc[3] * N3;
+        Hx += wc[2] * N2;
+        Hx += wc[1] * N1;
+        Hx += wc[0] * w0.c;
+        if (shift.y != (R)0) {  // B = C - i sigma K
+          horner_pm<R, 4, 5>(sTab + ct_off_K(ns) + seg * kCtK, u, wc);
+          const cx<R> q = wc[3] * N3 + wc[2] * N2 + wc[1] * N1 + wc[0] * w0.c;
+          Hx.x += shift.y * q.y;
+          Hx.y -= shift.y * q.x;
+        }
+        if (MODE == M_APPLY) {
+          out = Hx;
+        } else if (MODE == M_RESID) {
+          out = gv[P2] - Hx;
+        } else if (MODE == M_J2) {
+          out = xcv[P2] + a.omega_j * (dinvv[P2] * (gv[P2] - Hx));
+          if (Bs) out += Bs[idx];
+        } else {  // M_JSWEEP
+          out = xcv[P2] + a.omega_j * (DI[idx] * (gv[P2] - Hx));
+        }
       } else {
         R av[5];
         table_eval<R, 0, 5>(sTab, nseg, ds, inv_ds, eta_star(kap_prev), av);
@@ -471,22 +533,47 @@ __device__ __forceinline__ void fwd_body(const StencilCall<R>& a, int zblock, in
   }
 }
 
+// Weight tables of a launch in shared memory: the Hermite cubics, or (CW) the level's
+// combined quintics and transverse weights.  They travel by cp.async, with the first
+// plane's group: loads into registers stand before the march, and a block of 64
+// threads has eight of them per thread (residual of B on 39^3 in a graph: 13.6 us by
+// registers, 12.7 so).  The first barrier of the march makes them visible.
+template <bool CW>
+constexpr int tab_size() {
+  return CW ? (kCtCA + kCtK + kCtT) * (kMaxSeg + 1) : kMaxSeg * kNumFn * 4;
+}
+template <class R>
+__device__ __forceinline__ void copy_table(R* dst, const R* src, int n, int tid, int nth) {
+  constexpr int V = 16 / sizeof(R);  // (n is a multiple of V, both sides start on 16 bytes)
+  for (int i = tid * V; i < n; i += nth * V) cp_async<16>(dst + i, src + i, true);
+}
+template <bool CW, class R>
+__device__ __forceinline__ void load_table(const StencilCall<R>& a, R* sTab, int tid, int nth) {
+  if constexpr (CW) {
+    const int ns = a.tab.nseg + 1;
+    copy_table(sTab, a.lv.ctab, kCtCA * ns, tid, nth);
+    if (a.mass_shift.y != (R)0) copy_table(sTab + ct_off_K(ns), a.lv.ctab + ct_off_K(ns), kCtK * ns, tid, nth);
+    copy_table(sTab + ct_off_T(ns), a.lv.ctab + ct_off_T(ns), kCtT * ns, tid, nth);
+  } else {
+    copy_table(sTab, a.tab.coef, a.tab.nseg * kNumFn * 4, tid, nth);
+  }
+}
+
 // PATH 0: the PML-free rectangle (shell rows); 1: the PML frame around it
 // (general rows); 2: a whole (small) grid, the row form chosen per tile.
-template <class R, int MODE, int OP, int PATH>
+template <class R, int MODE, int OP, int PATH, bool CW>
 __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? (PATH == 0 ? 4 : 2) : 1) k_fwd(StencilCall<R> a, int zblock,
                                                                                       TileMap tm) {
   constexpr int PL = (PATH == 1) ? (TileW::PLN > TileT::PLN ? TileW::PLN : TileT::PLN) : TileSq::PLN;
   __shared__ __align__(16) cx<R> sX[NSTAGE * PL];
   __shared__ __align__(16) cx<R> sD[(MODE == M_J2) ? NSTAGE * PL : 1];
   __shared__ cx<R> sY1[(MODE == M_J2) ? PL : 1];
-  __shared__ __align__(16) R sTab[kMaxSeg * kNumFn * 4];
+  __shared__ __align__(16) R sTab[tab_size<CW>()];
   __shared__ R sKc[NSTAGE][NT];                                              // kappa of the own column
   __shared__ cx<R> sGc[(MODE == M_RESID || MODE == M_JSWEEP) ? NSTAGE : 1][NT];  // rhs of the own column
   __shared__ double sRed[32];
   const int tid = threadIdx.y * TX + threadIdx.x;
-  for (int i = tid; i < a.tab.nseg * kNumFn * 4; i += NT) sTab[i] = a.tab.coef[i];
-  // (visibility of sTab is ensured by the first __syncthreads of the march)
+  load_table<CW>(a, sTab, tid, NT);
   const int rhs = blockIdx.x % a.nrhs;
   const int t = blockIdx.x / a.nrhs;
   if constexpr (PATH == 1 && OP != OP_Q) {
@@ -496,21 +583,21 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? (PATH == 0 ? 4 : 2) : 1) 
       // strips below / above the rectangle: PML along y only away from the corners
       const bool xplain = f.x0 >= a.lv.plain_lo[0] && f.x0 + TileW::TXS - 1 <= a.lv.plain_hi[0];
       if (xplain)
-        fwd_body<R, MODE, OP, 3, TileW>(a, zblock, (int)blockIdx.z, tm, rhs, f.x0, f.y0, f.rx1, f.ry1, bid, sX, sD, sY1, sTab, sRed,
+        fwd_body<R, MODE, OP, 3, TileW, CW>(a, zblock, (int)blockIdx.z, tm, rhs, f.x0, f.y0, f.rx1, f.ry1, bid, sX, sD, sY1, sTab, sRed,
                                         sKc, sGc);
       else
-        fwd_body<R, MODE, OP, 2, TileW>(a, zblock, (int)blockIdx.z, tm, rhs, f.x0, f.y0, f.rx1, f.ry1, bid, sX, sD, sY1, sTab, sRed,
+        fwd_body<R, MODE, OP, 2, TileW, CW>(a, zblock, (int)blockIdx.z, tm, rhs, f.x0, f.y0, f.rx1, f.ry1, bid, sX, sD, sY1, sTab, sRed,
                                         sKc, sGc);
     } else {
       // strips left / right of the rectangle lie in its y range: PML along x only
-      fwd_body<R, MODE, OP, 1, TileT>(a, zblock, (int)blockIdx.z, tm, rhs, f.x0, f.y0, f.rx1, f.ry1, bid, sX, sD, sY1, sTab, sRed,
+      fwd_body<R, MODE, OP, 1, TileT, CW>(a, zblock, (int)blockIdx.z, tm, rhs, f.x0, f.y0, f.rx1, f.ry1, bid, sX, sD, sY1, sTab, sRed,
                                       sKc, sGc);
     }
   } else {
     const unsigned bid = (unsigned)(tm.bid_offset + t + tm.ntx * (blockIdx.y + gridDim.y * blockIdx.z));
     if constexpr (OP == OP_Q || PATH == 0) {
       const int x0 = tm.ox + t * TX, y0 = tm.oy + (int)blockIdx.y * TY;
-      fwd_body<R, MODE, OP, 0, TileSq>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab, sRed,
+      fwd_body<R, MODE, OP, 0, TileSq, CW>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab, sRed,
                                        sKc, sGc);
     } else {
       constexpr int GX = TileG::TXS, GY = TileG::TYS;
@@ -519,10 +606,10 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? (PATH == 0 ? 4 : 2) : 1) 
       const bool plain = (x0 >= L.plain_lo[0]) && (x0 + GX - 1 <= L.plain_hi[0]) && (y0 >= L.plain_lo[1]) &&
                          (y0 + GY - 1 <= L.plain_hi[1]);
       if (plain)
-        fwd_body<R, MODE, OP, 0, TileG>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab, sRed,
+        fwd_body<R, MODE, OP, 0, TileG, CW>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab, sRed,
                                         sKc, sGc);
       else
-        fwd_body<R, MODE, OP, 2, TileG>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab, sRed,
+        fwd_body<R, MODE, OP, 2, TileG, CW>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab, sRed,
                                         sKc, sGc);
     }
   }
@@ -532,17 +619,17 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? (PATH == 0 ? 4 : 2) : 1) 
 // A whole very small grid: 8 x 8 tiles of 64 threads.  A 256-thread tile puts a
 // 13^3 grid on 7 of 152 SMs, and in double precision a tile-plane takes an SM's two
 // FP64 lanes some 10 thousand cycles.
-template <class R, int MODE, int OP>
+template <class R, int MODE, int OP, bool CW>
 __global__ void __launch_bounds__(TileS::NTH) k_fwd_small(StencilCall<R> a, int zblock, TileMap tm) {
   constexpr int PL = TileS::PLN, NTS = TileS::NTH;
   __shared__ __align__(16) cx<R> sX[NSTAGE * PL];
   __shared__ __align__(16) cx<R> sD[(MODE == M_J2) ? NSTAGE * PL : 1];
   __shared__ cx<R> sY1[(MODE == M_J2) ? PL : 1];
-  __shared__ __align__(16) R sTab[kMaxSeg * kNumFn * 4];
+  __shared__ __align__(16) R sTab[tab_size<CW>()];
   __shared__ R sKc[NSTAGE][NTS];
   __shared__ cx<R> sGc[(MODE == M_RESID || MODE == M_JSWEEP) ? NSTAGE : 1][NTS];
   __shared__ double sRed[32];
-  for (int i = threadIdx.x; i < a.tab.nseg * kNumFn * 4; i += NTS) sTab[i] = a.tab.coef[i];
+  load_table<CW>(a, sTab, (int)threadIdx.x, NTS);
   const int rhs = blockIdx.x % a.nrhs, t = blockIdx.x / a.nrhs;
   const unsigned bid = (unsigned)(t + tm.ntx * (blockIdx.y + gridDim.y * blockIdx.z));
   const int x0 = t * TileS::TXS, y0 = (int)blockIdx.y * TileS::TYS;
@@ -550,10 +637,10 @@ __global__ void __launch_bounds__(TileS::NTH) k_fwd_small(StencilCall<R> a, int 
   const bool plain = OP == OP_Q || (x0 >= L.plain_lo[0] && x0 + TileS::TXS - 1 <= L.plain_hi[0] &&
                                     y0 >= L.plain_lo[1] && y0 + TileS::TYS - 1 <= L.plain_hi[1]);
   if (plain)
-    fwd_body<R, MODE, OP, 0, TileS>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab,
+    fwd_body<R, MODE, OP, 0, TileS, CW>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab,
                                     sRed, sKc, sGc);
   else if constexpr (OP != OP_Q)
-    fwd_body<R, MODE, OP, 2, TileS>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab,
+    fwd_body<R, MODE, OP, 2, TileS, CW>(a, zblock, (int)blockIdx.z, tm, rhs, x0, y0, tm.rx1, tm.ry1, bid, sX, sD, sY1, sTab,
                                     sRed, sKc, sGc);
 }
 
@@ -644,7 +731,7 @@ static FwdPlan plan_fwd(const LevelView<R>& L, int nrhs, int op) {
   return plan_layout(L.nx, L.ny, L.nz, L.plain_lo, L.plain_hi, op, zb, L.zblock_f);
 }
 
-template <class R, int MODE, int OP>
+template <class R, int MODE, int OP, bool CW = false>
 static void launch_fwd_t(const StencilCall<R>& c, cudaStream_t s) {
   const LevelView<R>& L = c.lv;
   const FwdPlan p = plan_fwd(L, c.nrhs, OP);
@@ -658,10 +745,10 @@ static void launch_fwd_t(const StencilCall<R>& c, cudaStream_t s) {
     dim3 grid(p.TXT * c.nrhs, p.TYT, p.nzb);
     count_launch();
     if (p.small) {
-      k_fwd_small<R, MODE, OP><<<grid, TileS::NTH, 0, s>>>(c, p.zb, tm);
+      k_fwd_small<R, MODE, OP, CW><<<grid, TileS::NTH, 0, s>>>(c, p.zb, tm);
       return;
     }
-    k_fwd<R, MODE, OP, (OP == OP_Q) ? 0 : 2><<<grid, dim3(TX, TY), 0, s>>>(c, p.zb, tm);
+    k_fwd<R, MODE, OP, (OP == OP_Q) ? 0 : 2, CW><<<grid, dim3(TX, TY), 0, s>>>(c, p.zb, tm);
     return;
   }
   TileMap ti;
@@ -684,10 +771,10 @@ static void launch_fwd_t(const StencilCall<R>& c, cudaStream_t s) {
     cudaStreamWaitEvent(s2, c.fork, 0);
   }
   count_launch();
-  k_fwd<R, MODE, OP, 0><<<dim3(p.RW * c.nrhs, p.RH, p.nzb), dim3(TX, TY), 0, s>>>(c, p.zb, ti);
+  k_fwd<R, MODE, OP, 0, CW><<<dim3(p.RW * c.nrhs, p.RH, p.nzb), dim3(TX, TY), 0, s>>>(c, p.zb, ti);
   if (tp.count > 0) {
     count_launch();
-    k_fwd<R, MODE, OP, 1><<<dim3(tp.count * c.nrhs, 1, p.nzbf), dim3(TX, TY), 0, s2>>>(c, p.zbf, tp);
+    k_fwd<R, MODE, OP, 1, CW><<<dim3(tp.count * c.nrhs, 1, p.nzbf), dim3(TX, TY), 0, s2>>>(c, p.zbf, tp);
   }
   if (fork) {
     cudaEventRecord(c.join, s2);
@@ -785,18 +872,28 @@ long long replay_gather_layout(int nx, int ny, int nz, const int* plo, const int
   return bad;
 }
 
+template <class R, bool CW>
+static void launch_fwd_ab(const StencilCall<R>& c, int mode, cudaStream_t s) {
+  switch (mode) {
+    case M_APPLY: launch_fwd_t<R, M_APPLY, OP_AB, CW>(c, s); break;
+    case M_RESID: launch_fwd_t<R, M_RESID, OP_AB, CW>(c, s); break;
+    case M_J2: launch_fwd_t<R, M_J2, OP_AB, CW>(c, s); break;
+    case M_JSWEEP: launch_fwd_t<R, M_JSWEEP, OP_AB, CW>(c, s); break;
+  }
+}
 template <class R>
 void launch_fwd_gather(const StencilCall<R>& c, int mode, int op, cudaStream_t s) {
   if (op == OP_Q) {
     launch_fwd_t<R, M_APPLY, OP_Q>(c, s);
     return;
   }
-  switch (mode) {
-    case M_APPLY: launch_fwd_t<R, M_APPLY, OP_AB>(c, s); break;
-    case M_RESID: launch_fwd_t<R, M_RESID, OP_AB>(c, s); break;
-    case M_J2: launch_fwd_t<R, M_J2, OP_AB>(c, s); break;
-    case M_JSWEEP: launch_fwd_t<R, M_JSWEEP, OP_AB>(c, s); break;
+  if constexpr (sizeof(R) == sizeof(float)) {
+    if (c.lv.level == 0) {
+      launch_fwd_ab<R, true>(c, mode, s);
+      return;
+    }
   }
+  launch_fwd_ab<R, false>(c, mode, s);
 }
 
 template void launch_fwd_gather<float>(const StencilCall<float>&, int, int, cudaStream_t);

@@ -63,19 +63,33 @@ using CoreT = Tile<32, 2, NPY>;  // 64 x 8 or 64 x 4
 
 // Coefficient tables of a level (single precision), NS = nseg + 1 segments, the
 // last one the clamp eta >= 0.4, in the local coordinate u = eta / ds - segment:
-//   C: C_0..C_3 of A, quintics, [segment][power][4]
-//   F: alpha_4, alpha_5 and the mass weights M_0..M_3, cubics, [segment][power][6]
 //   Q: shell weights of Q_h, cubics, [segment][power][4]
-//   S: C_0..C_3 of A again, as the interpolating cubics of nsub equal parts of
-//      each segment (u in parts), [part][power][4]; the clamp is the last part.
-//      After them alpha_4, alpha_5 in the same parts, [power][2].  nsub is the
-//      smallest that reproduces the quintics to kSubTol of the row's largest
-//      weight: 4 with the shipped table (3e-9, a sixteenth of a single-precision
-//      ulp), more with a coarser one, up to kMaxParts parts in all.
-constexpr int kMtC = 24, kMtF = 24, kMtQ = 16, kMtS = 24, kMaxParts = 512;
+//   F: alpha_4 - 3/4, alpha_5 - 1/4 and the mass weights M_0..M_3, cubics,
+//      [segment][power][6].  The offsets keep the two alphas small, and the stiffness
+//      weights that B forms from them (6 alpha_4 most of all) accurate: random fields,
+//      interior rows, 5.4e-8 of the norm against 7.2e-8 with the alphas themselves.
+//   S: C_0..C_3 of A (stiffness and mass weights combined), as the interpolating
+//      cubics of nsub equal parts of each segment (u in parts), [part][power][4]; the
+//      clamp is the last part.  After them alpha_4, alpha_5 in the same parts,
+//      [power][2].  nsub is the smallest that reproduces the quintics, which C is
+//      exactly, to kSubTol of the row's largest weight: 4 with the shipped table
+//      (4e-10; 2 leave 7e-9), more with a coarser one, up to kMaxParts parts in all.
+// B evaluates L - (1 + i sigma) kappa^2 M from F.  Taking C from S there (5.4e-8 too)
+// costs a fifth of the 2h level's time, 41.7 -> 49.9 us for J_2 on 145^3: two more
+// 128-bit table loads per node, and 65 parts where F has 17 rows.
+constexpr int kMtQ = 16, kMtF = 24, kMtS = 24, kMaxParts = 512;
 constexpr double kSubTol = 6e-9;
-__host__ __device__ constexpr int mt_off_S(int ns) { return (kMtC + kMtF + kMtQ) * ns; }
+constexpr double kA4Off = 0.75, kA5Off = 0.25;  // offsets of table F
+__host__ __device__ constexpr int mt_off_F(int ns) { return kMtQ * ns; }
+__host__ __device__ constexpr int mt_off_S(int ns) { return (kMtQ + kMtF) * ns; }
 __host__ __device__ constexpr int mt_size(int ns) { return mt_off_S(ns) + kMtS * (kMaxParts + 1); }
+// The table of an operator kind (A: S, B: F, Q): its place, and floats per row.
+template <int OPK>
+__host__ __device__ constexpr int tab_off(int ns) {
+  return OPK == OPK_A ? mt_off_S(ns) : OPK == OPK_B ? mt_off_F(ns) : 0;
+}
+template <int OPK>
+constexpr int kTabRow = OPK == OPK_A ? kMtS : OPK == OPK_B ? kMtF : kMtQ;
 
 template <int MODE, class TL, int RB>
 struct Smem {
@@ -85,9 +99,8 @@ struct Smem {
   static constexpr int PREF = MODE == M_J2 ? 3 : 5;
   static constexpr size_t a16(size_t x) { return (x + 15) & ~(size_t)15; }
   static constexpr size_t o_d = a16((size_t)NSTG * RB * TL::PLN * 8);
-  static constexpr size_t o_tab = a16(o_d + (MODE == M_J2 ? (size_t)NSTG * TL::PLN * 8 : 0));
-  static constexpr size_t o_red = a16(o_tab + (size_t)24 * (kMaxSeg + 1) * 4);
-  static constexpr size_t bytes = o_red + 32 * sizeof(double);
+  static constexpr size_t o_red = a16(o_d + (MODE == M_J2 ? (size_t)NSTG * TL::PLN * 8 : 0));
+  static constexpr size_t o_tab = o_red + 32 * sizeof(double);  // sized at the launch
 };
 
 // Blocks of a launch, in this order: the z-PML slabs (whole x-y range, general
@@ -171,46 +184,54 @@ __device__ __forceinline__ float2 row_value(const float* w, float k2, float inv_
     N2 = add2(s.p2, n.e);
   }
   const float2 N3 = add2(s.p3, n.k);
-  float2 h = make_float2(w[0] * s.c.x, w[0] * s.c.y);
-  rfma(h, w[1], N1);
-  rfma(h, w[2], N2);
-  rfma(h, w[3], N3);
-  if constexpr (OPK == OPK_B) {
-    // w[4..7]: mass weights; H = ell^-2 (L - (1 + i sigma) kappa^2 M)
-    float2 q = make_float2(w[4] * s.c.x, w[4] * s.c.y);
-    rfma(q, w[5], N1);
-    rfma(q, w[6], N2);
-    rfma(q, w[7], N3);
-    q.x *= k2;
-    q.y *= k2;
-    h.x = inv_l2 * (h.x - q.x + sigma * q.y);
-    h.y = inv_l2 * (h.y - q.y - sigma * q.x);
-  }
-  if constexpr (CORR || ZP) {
+  // Terms are added smallest first (PML corrections, corners inwards): only the last
+  // addition then rounds at the size of the centre's term.
+  [[maybe_unused]] float2 cor = make_float2(0.f, 0.f);
+  if constexpr (CORR) {
     const float q5 = 0.25f * a5, qb = fmaf(-0.25f, a4 + a5, 0.25f);
-    if constexpr (CORR) {
-      rfma(h, a4, s.A);
-      rfma(h, q5, add2(s.BA, nA));
-      rfma(h, qb, add2(s.Bm, nB));
-      s.BA = add2(nB, s.A);
-      s.Bm = s.B;
-      s.A = nA;
-      s.B = nB;
-    }
+    const float2 A1 = add2(s.BA, nA), B1 = add2(s.Bm, nB);
+    cor = make_float2(qb * B1.x, qb * B1.y);
+    rfma(cor, q5, A1);
+    rfma(cor, a4, s.A);
+    s.BA = add2(nB, s.A);
+    s.Bm = s.B;
+    s.A = nA;
+    s.B = nB;
     if constexpr (ZP) {
       if (zp) {  // eps+ T(n - o) + eps- T(m - o), T the transverse-weighted sum
         float2 t = make_float2(0.f, 0.f);
-        rfma(t, a4, sub2(n.c, s.c));
-        rfma(t, q5, sub2(n.e, s.e));
         rfma(t, qb, sub2(n.k, s.k));
-        cfma2(h, ezp, t);
+        rfma(t, q5, sub2(n.e, s.e));
+        rfma(t, a4, sub2(n.c, s.c));
+        cfma2(cor, ezp, t);
         t = make_float2(0.f, 0.f);
-        rfma(t, a4, sub2(s.p1, s.c));
-        rfma(t, q5, sub2(s.p2, s.e));
         rfma(t, qb, sub2(s.p3, s.k));
-        cfma2(h, ezm, t);
+        rfma(t, q5, sub2(s.p2, s.e));
+        rfma(t, a4, sub2(s.p1, s.c));
+        cfma2(cor, ezm, t);
       }
     }
+  }
+  float2 h;
+  if constexpr (OPK != OPK_B && CORR) {
+    h = cor;
+    rfma(h, w[3], N3);
+  } else {
+    h = make_float2(w[3] * N3.x, w[3] * N3.y);
+  }
+  rfma(h, w[2], N2);
+  rfma(h, w[1], N1);
+  rfma(h, w[0], s.c);
+  if constexpr (OPK == OPK_B) {
+    // w[4..7]: mass weights; H = ell^-2 (L - (1 + i sigma) kappa^2 M)
+    float2 q = make_float2(w[7] * N3.x, w[7] * N3.y);
+    rfma(q, w[6], N2);
+    rfma(q, w[5], N1);
+    rfma(q, w[4], s.c);
+    const float k2s = sigma * k2;
+    const float hx = fmaf(k2s, q.y, fmaf(-k2, q.x, h.x)), hy = fmaf(-k2s, q.x, fmaf(-k2, q.y, h.y));
+    h.x = CORR ? fmaf(inv_l2, hx, cor.x) : inv_l2 * hx;
+    h.y = CORR ? fmaf(inv_l2, hy, cor.y) : inv_l2 * hy;
   }
   if constexpr (ZP) {
     s.p1 = s.c;
@@ -226,19 +247,92 @@ __device__ __forceinline__ float2 row_value(const float* w, float k2, float inv_
   return h;
 }
 
-// the six functions of table F at segment seg (power-major, 24 floats, 16-byte aligned)
-__device__ __forceinline__ void eval_f6(const float* t, float u, float* f) {
-  float c[24];
+__device__ __forceinline__ float4 lds128(unsigned a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ float2 lds64(unsigned a) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ float lds32(unsigned a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+  return v;
+}
+// Rows of the launch's table, without the clamp, and its segments.
+template <int OPK>
+__device__ __forceinline__ int tab_rows(const StencilCall<float>& a) {
+  return a.tab.nseg * (OPK == OPK_A ? a.lv.nsub : 1);
+}
+template <int OPK>
+__device__ __forceinline__ SegK tab_seg(const StencilCall<float>& a) {
+  SegK K;
+  K.s1 = a.tab.inv_ds * (float)kInv2Pi * (OPK == OPK_A ? (float)a.lv.nsub : 1.f);
+  K.hi = (float)tab_rows<OPK>(a);
+  K.sc = K.s1 / K.hi;
+  K.off = -0.5f / K.hi;
+  return K;
+}
+template <int OPK>
+__device__ __forceinline__ void load_table(const StencilCall<float>& a, unsigned char* dst) {
+  const float4* g = reinterpret_cast<const float4*>(a.lv.mtab + tab_off<OPK>(a.tab.nseg + 1));
+  float4* t = reinterpret_cast<float4*>(dst);
+  for (int i = threadIdx.x; i < kTabRow<OPK> / 4 * (tab_rows<OPK>(a) + 1); i += NT) t[i] = g[i];
+}
+// Weights of a row: 4 of A or Q, 4 stiffness and 4 mass weights of B; with T also
+// alpha_4 and alpha_5.
+template <int OPK, bool T = false>
+__device__ __forceinline__ void row_weights(const SegK& K, unsigned tab, float kap, float* w, float* a45 = nullptr) {
+  float u;
+  const unsigned t = tab + 4u * kTabRow<OPK> * (unsigned)seg_u(K, kap, u);
+  if constexpr (OPK != OPK_B) {
+    const float4 c3 = lds128(t + 48), c2 = lds128(t + 32), c1 = lds128(t + 16), c0 = lds128(t);
+    w[0] = fmaf(fmaf(fmaf(c3.x, u, c2.x), u, c1.x), u, c0.x);
+    w[1] = fmaf(fmaf(fmaf(c3.y, u, c2.y), u, c1.y), u, c0.y);
+    w[2] = fmaf(fmaf(fmaf(c3.z, u, c2.z), u, c1.z), u, c0.z);
+    w[3] = fmaf(fmaf(fmaf(c3.w, u, c2.w), u, c1.w), u, c0.w);
+    if constexpr (T) {
+      const float4 lo = lds128(t + 64), hi = lds128(t + 80);
+      a45[0] = fmaf(fmaf(fmaf(hi.z, u, hi.x), u, lo.z), u, lo.x);
+      a45[1] = fmaf(fmaf(fmaf(hi.w, u, hi.y), u, lo.w), u, lo.y);
+    }
+  } else {
+    float c[24], f[6];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const float4 v = reinterpret_cast<const float4*>(t)[i];
-    c[4 * i] = v.x;
-    c[4 * i + 1] = v.y;
-    c[4 * i + 2] = v.z;
-    c[4 * i + 3] = v.w;
+    for (int i = 0; i < 6; ++i) {
+      const float4 v = lds128(t + 16 * i);
+      c[4 * i] = v.x;
+      c[4 * i + 1] = v.y;
+      c[4 * i + 2] = v.z;
+      c[4 * i + 3] = v.w;
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) f[i] = fmaf(fmaf(fmaf(c[18 + i], u, c[12 + i]), u, c[6 + i]), u, c[i]);
+    // 6 a4, a5 - a4, (1 - a4) / 2 - a5, 3 (a4 + a5 - 1) / 4 of a4 = f0 + 3/4, a5 = f1 + 1/4
+    w[0] = fmaf(6.f, f[0], 4.5f);
+    w[1] = (f[1] - f[0]) - 0.5f;
+    w[2] = fmaf(-0.5f, f[0], -0.125f) - f[1];
+    w[3] = 0.75f * (f[0] + f[1]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w[4 + q] = f[2 + q];
+    if constexpr (T) {
+      a45[0] = f[0] + (float)kA4Off;
+      a45[1] = f[1] + (float)kA5Off;
+    }
   }
-#pragma unroll
-  for (int i = 0; i < 6; ++i) f[i] = fmaf(fmaf(fmaf(c[18 + i], u, c[12 + i]), u, c[6 + i]), u, c[i]);
+}
+
+// The two-sweep Jacobi map of a row: with y1 = omega D^-1 g and c = y1 / omega,
+// y1 + omega D^-1 (g - H y1) = omega (2 c - omega D^-1 H c); d = 1/diag, h = H c.
+// Rounding c to single precision is what rounding g once would do to the result.
+// Reading g again for the residual itself takes that out (289^3 9.5e-8 -> 9.05e-8 of
+// the norm) and costs 14 % (226 -> 258 us): the planes hold c by then.
+__device__ __forceinline__ float2 jacobi2(float om, float2 d, float2 c, float2 h) {
+  const float tx = d.x * h.x - d.y * h.y, ty = d.x * h.y + d.y * h.x;
+  return make_float2(om * fmaf(-om, tx, c.x + c.x), om * fmaf(-om, ty, c.y + c.y));
 }
 
 // Sum of nrm2 over the launch's blocks for each right-hand side of this block:
@@ -276,13 +370,11 @@ __device__ __forceinline__ void tile_body(const StencilCall<float>& a, unsigned 
                                           int y0, int rx1, int ry1, int rhs0, unsigned bid, unsigned nblk) {
   using SM = Smem<MODE, TL, RB>;
   constexpr int NSTG = SM::NSTG, PREF = SM::PREF, PW = TL::PW, PLN = TL::PLN, NSLOT = TL::NSLOT, NPX = TL::NPX, NPY = TL::NPY;
-  constexpr bool TC = OPK == OPK_A, TQ = OPK == OPK_Q;  // tables C, Q or (B) F
-
   const LevelView<float>& L = a.lv;
   cx<float>* sX = reinterpret_cast<cx<float>*>(smem);
   cx<float>* sD = reinterpret_cast<cx<float>*>(smem + SM::o_d);
-  float* sT = reinterpret_cast<float*>(smem + SM::o_tab);
   double* sRed = reinterpret_cast<double*>(smem + SM::o_red);
+  const unsigned tab = (unsigned)__cvta_generic_to_shared(smem + SM::o_tab);
 
   const int tid = threadIdx.x;
   const int tx = tid % TL::TXT, ty = tid / TL::TXT;
@@ -290,17 +382,8 @@ __device__ __forceinline__ void tile_body(const StencilCall<float>& a, unsigned 
   const int nplanes = zb1 - zb0 + 2;
   const long long plane = (long long)nx * ny;
   const long long xs = a.xstride > 0 ? a.xstride : L.N, ys = a.ystride > 0 ? a.ystride : L.N;
-  const int ns = a.tab.nseg + 1;
-  SegK K;
-  K.s1 = a.tab.inv_ds * (float)kInv2Pi;
-  K.hi = (float)a.tab.nseg;
-  K.sc = K.s1 / K.hi;
-  K.off = -0.5f / K.hi;
-
-  {
-    const int off = TC ? 0 : (TQ ? (kMtC + kMtF) * ns : kMtC * ns), per = TQ ? kMtQ : 24;
-    for (int i = tid; i < per * ns; i += NT) sT[i] = L.mtab[off + i];
-  }
+  const SegK K = tab_seg<OPK>(a);
+  load_table<OPK>(a, smem + SM::o_tab);
 
   // this thread's columns: (gx0 + i, gy0 + j); addresses are clamped into the
   // grid (a value one past a row's end is read from kappa and 1/diag, which are
@@ -498,25 +581,11 @@ __device__ __forceinline__ void tile_body(const StencilCall<float>& a, unsigned 
           n.e = add2(hx[j + 1][i], add2(v[j][i + 1], v[j + 2][i + 1]));
           n.k = add2(hx[j][i], hx[j + 2][i]);
           // the row's weights (before the first row completes: of a row nobody stores)
-          const float kap = kq[V][j][i], k2 = kap * kap;
-          float u, wt[8];
-          const int seg = seg_u(K, kap, u);
-          if constexpr (TC) {
-            horner_pm<float, 4, 5>(sT + seg * kMtC, u, wt);
-          } else if constexpr (TQ) {
-            horner_pm<float, 4, 3>(sT + seg * kMtQ, u, wt);
-          } else {
-            float f[6];
-            eval_f6(sT + seg * kMtF, u, f);
-            wt[0] = 6.f * f[0];
-            wt[1] = f[1] - f[0];
-            wt[2] = fmaf(-0.5f, f[0], 0.5f) - f[1];
-            wt[3] = fmaf(0.75f, f[0] + f[1], -0.75f);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) wt[4 + q] = f[2 + q];
-          }
+          const float kap = kq[V][j][i];
+          float wt[8];
+          row_weights<OPK>(K, tab, kap, wt);
           [[maybe_unused]] const float2 oc = w[r][j][i].c;  // the row's own value
-          const float2 h = row_value<OPK, false, false>(wt, k2, inv_l2, sigma, w[r][j][i], n, n.c, n.c, false, n.c, n.c,
+          const float2 h = row_value<OPK, false, false>(wt, kap * kap, inv_l2, sigma, w[r][j][i], n, n.c, n.c, false, n.c, n.c,
                                                         0.f, 0.f);
           if (fin) {
             float2 out;
@@ -526,14 +595,10 @@ __device__ __forceinline__ void tile_body(const StencilCall<float>& a, unsigned 
               out = make_float2(gq[V][r][j][i].x - h.x, gq[V][r][j][i].y - h.y);
               if (act[j][i]) nrm2[r] = fmaf(out.x, out.x, fmaf(out.y, out.y, nrm2[r]));
             } else {
-              // with y1 = omega D^-1 g and c = y1 / omega:
-              // y1 + omega D^-1 (g - H y1) = omega (2 c - omega D^-1 H c)
               const cx<float> d = MODE == M_J2 ? sD[stp * PLN + (NPY * ty + j + 1) * PW + NPX * tx + i + 1]
                                                : a.dinv[p * plane + col[j] + i];
               if constexpr (MODE == M_J2) {
-                const float wx = om * d.x, wy = om * d.y;
-                out.x = om * (2.f * oc.x - (wx * h.x - wy * h.y));
-                out.y = om * (2.f * oc.y - (wx * h.y + wy * h.x));
+                out = jacobi2(om, make_float2(d.x, d.y), oc, h);
                 out.x += gq[V][r][j][i].x;
                 out.y += gq[V][r][j][i].y;
               } else {
@@ -616,11 +681,11 @@ __device__ __forceinline__ bool mbar_try(unsigned b, unsigned ph) {
 // Bounded wait (polls: 64 ns apart).  Once one has given up the thread waits no
 // more (dead, the planes asked for by then): the kernel ends with invalid results
 // and the host reports it.
-__device__ __forceinline__ void mbar_wait(unsigned b, unsigned ph, int& dead, int armed, int* err, unsigned polls) {
+__device__ __forceinline__ void mbar_wait(unsigned b, unsigned ph, int& dead, int armed, const StencilCall<float>& a) {
   if (dead) return;
-  for (int i = 0; i < 16; ++i)
+  for (int i = 0; i < 4; ++i)
     if (mbar_try(b, ph)) return;  // (suspends for a while by itself)
-  for (unsigned i = 0; i < polls; ++i) {
+  for (unsigned i = 0; i < a.polls; ++i) {
     unsigned ok;
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
@@ -631,73 +696,14 @@ __device__ __forceinline__ void mbar_wait(unsigned b, unsigned ph, int& dead, in
     __nanosleep(64);
   }
   dead = armed;
-  if (err) atomicExch(err, 1);
+  if (a.err) atomicExch(a.err, 1);
 }
 template <int BYTES>
 __device__ __forceinline__ void cp_s(unsigned dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(dst), "l"(src), "n"(BYTES));
 }
-__device__ __forceinline__ float4 lds128(unsigned a) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ float2 lds64(unsigned a) {
-  float2 v;
-  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ float lds32(unsigned a) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
-  return v;
-}
 __device__ __forceinline__ void sts64(unsigned a, float2 v) {
   asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y));
-}
-
-// weights of a row: 4 of A (cubics on the sub-segments), or 4 stiffness and 4
-// mass weights of B; with T also alpha_4 and alpha_5
-template <int OPK, bool T = false>
-__device__ __forceinline__ void core_weights(const SegK& K, unsigned tab, float kap, float* wt, float* a45 = nullptr) {
-  float u;
-  const int seg = seg_u(K, kap, u);
-  if constexpr (OPK == OPK_A) {
-    const unsigned t = tab + 4u * kMtS * (unsigned)seg;
-    const float4 c3 = lds128(t + 48), c2 = lds128(t + 32), c1 = lds128(t + 16), c0 = lds128(t);
-    wt[0] = fmaf(fmaf(fmaf(c3.x, u, c2.x), u, c1.x), u, c0.x);
-    wt[1] = fmaf(fmaf(fmaf(c3.y, u, c2.y), u, c1.y), u, c0.y);
-    wt[2] = fmaf(fmaf(fmaf(c3.z, u, c2.z), u, c1.z), u, c0.z);
-    wt[3] = fmaf(fmaf(fmaf(c3.w, u, c2.w), u, c1.w), u, c0.w);
-    if constexpr (T) {
-      const float4 lo = lds128(t + 64), hi = lds128(t + 80);
-      a45[0] = fmaf(fmaf(fmaf(hi.z, u, hi.x), u, lo.z), u, lo.x);
-      a45[1] = fmaf(fmaf(fmaf(hi.w, u, hi.y), u, lo.w), u, lo.y);
-    }
-  } else {
-    const unsigned t = tab + 96u * (unsigned)seg;
-    float c[24], f[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      const float4 v = lds128(t + 16 * i);
-      c[4 * i] = v.x;
-      c[4 * i + 1] = v.y;
-      c[4 * i + 2] = v.z;
-      c[4 * i + 3] = v.w;
-    }
-#pragma unroll
-    for (int i = 0; i < 6; ++i) f[i] = fmaf(fmaf(fmaf(c[18 + i], u, c[12 + i]), u, c[6 + i]), u, c[i]);
-    wt[0] = 6.f * f[0];
-    wt[1] = f[1] - f[0];
-    wt[2] = fmaf(-0.5f, f[0], 0.5f) - f[1];
-    wt[3] = fmaf(0.75f, f[0] + f[1], -0.75f);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) wt[4 + q] = f[2 + q];
-    if constexpr (T) {
-      a45[0] = f[0];
-      a45[1] = f[1];
-    }
-  }
 }
 
 __device__ __forceinline__ void tma_box(unsigned dst, const CUtensorMap* m, int c0, int c1, unsigned bar) {
@@ -714,26 +720,16 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
                                           unsigned nblk) {
   using SM = CoreSmem<MODE, NPY, RB>;
   constexpr int NSTG = SM::NSTG, PREF = SM::PREF, XR = SM::XR;
-  constexpr bool J2 = SM::J2, OWN = SM::OWN, TC = OPK == OPK_A;
-  constexpr int NW = TC ? 4 : 8;
+  constexpr bool J2 = SM::J2, OWN = SM::OWN;
+  constexpr int NW = OPK == OPK_A ? 4 : 8;
   const LevelView<float>& L = a.lv;
   const unsigned sb = (unsigned)__cvta_generic_to_shared(smem);
   const int tid = threadIdx.x, lane = tid & 31, ty = tid >> 5;
   const int nx = L.nx, nplanes = zb1 - zb0 + 2;
   const long long plane = (long long)nx * L.ny;
   const long long ys = a.ystride > 0 ? a.ystride : L.N;
-  SegK K;
-  const int nq = a.tab.nseg * (TC ? L.nsub : 1);
-  K.s1 = a.tab.inv_ds * (float)kInv2Pi * (TC ? (float)L.nsub : 1.f);
-  K.hi = (float)nq;
-  K.sc = K.s1 / K.hi;
-  K.off = -0.5f / K.hi;
-  {
-    const int ns = a.tab.nseg + 1;
-    const float4* g = reinterpret_cast<const float4*>(L.mtab + (TC ? mt_off_S(ns) : kMtC * ns));
-    float4* t = reinterpret_cast<float4*>(smem + SM::o_tab);
-    for (int i = tid; i < 6 * (nq + 1); i += NT) t[i] = g[i];
-  }
+  const SegK K = tab_seg<OPK>(a);
+  load_table<OPK>(a, smem + SM::o_tab);
   const unsigned full = sb + SM::o_bar, empty = full + 8 * NSTG, tab = sb + SM::o_tab;
   if (tid == 0) {
 #pragma unroll
@@ -865,7 +861,7 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
   int st = 0;
   unsigned ph = 0;
   if constexpr (J2) {
-    mbar_wait(full, 0, dead, min(PREF, nplanes), a.err, a.polls);
+    mbar_wait(full, 0, dead, min(PREF, nplanes), a);
     transform(0, 0);
   }
 
@@ -882,17 +878,17 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
       if (tid == 0 && k + PREF < nplanes && !dead) fetch(k + PREF, s2);
       const int sn = st + 1 == NSTG ? 0 : st + 1;
       if (k + 1 < nplanes) {
-        mbar_wait(full + 8 * sn, ph ^ (sn == 0), dead, min(k + PREF + 1, nplanes), a.err, a.polls);
+        mbar_wait(full + 8 * sn, ph ^ (sn == 0), dead, min(k + PREF + 1, nplanes), a);
         transform(k + 1, sn);
       }
     } else {
       if (tid == 0 && k + PREF < nplanes) {
         if (k + PREF >= NSTG)
-          mbar_wait(empty + 8 * s2, (unsigned)((k + PREF) / NSTG - 1) & 1, dead, k + PREF, a.err, a.polls);
+          mbar_wait(empty + 8 * s2, (unsigned)((k + PREF) / NSTG - 1) & 1, dead, k + PREF, a);
         if (!dead) fetch(k + PREF, s2);
       }
       __syncwarp();
-      mbar_wait(full + 8 * st, ph, dead, min(k + PREF + 1, nplanes), a.err, a.polls);
+      mbar_wait(full + 8 * st, ph, dead, min(k + PREF + 1, nplanes), a);
     }
     // what the Jacobi map is added to (a ring for it would cost a block per SM)
     [[maybe_unused]] float2 bq[RB][NPY][2];
@@ -923,8 +919,8 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
     }
     float wt2[RB > 1 ? 2 : 1][NW];
     if constexpr (RB > 1) {
-      core_weights<OPK>(K, tab, kap[0][0], wt2[0]);
-      core_weights<OPK>(K, tab, kap[0][1], wt2[1]);
+      row_weights<OPK>(K, tab, kap[0][0], wt2[0]);
+      row_weights<OPK>(K, tab, kap[0][1], wt2[1]);
     }
 #pragma unroll
     for (int r = 0; r < RB; ++r) {
@@ -963,11 +959,11 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
           n.e = add2(hx[j + 1][i], add2(v[j][i + 1], v[j + 2][i + 1]));
           n.k = add2(hx[j][i], hx[j + 2][i]);
           float wt1[NW];
-          if constexpr (RB == 1) core_weights<OPK>(K, tab, kap[j][i], wt1);
+          if constexpr (RB == 1) row_weights<OPK>(K, tab, kap[j][i], wt1);
           const float* wt = RB == 1 ? wt1 : wt2[RB == 1 ? 0 : i];
           [[maybe_unused]] const float2 oc = w[r][j][i].c;
-          const float2 h = row_value<OPK, false, false>(wt, kap[j][i] * kap[j][i], inv_l2, sigma, w[r][j][i], n, n.c,
-                                                        n.c, false, n.c, n.c, 0.f, 0.f);
+          const float2 h = row_value<OPK, false, false>(wt, kap[j][i] * kap[j][i], inv_l2, sigma, w[r][j][i], n, n.c, n.c,
+                                                        false, n.c, n.c, 0.f, 0.f);
           if (fin) {
             float2 out = h;
             if constexpr (MODE == M_RESID || MODE == M_JSWEEP) {
@@ -979,14 +975,10 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
                 out = make_float2(fmaf(om, d.x * out.x - d.y * out.y, oc.x), fmaf(om, d.x * out.y + d.y * out.x, oc.y));
               }
             } else if constexpr (J2) {
-              // with y1 = omega D^-1 g and c = y1 / omega:
-              // y1 + omega D^-1 (g - H y1) = omega (2 c - omega D^-1 H c)
               const int sp = st == 0 ? NSTG - 1 : st - 1;
               const unsigned di = (unsigned)((rowd + (k - 1) * L.ny + NPY * ty + j + 1) * nx + x0 - 1) & 1;
               const float2 d = lds64(sb + sp * SM::stage + SM::o_d + xo[j + 1] + 8 * (di + 1 + i));
-              const float wx = om * d.x, wy = om * d.y;
-              out.x = om * (2.f * oc.x - (wx * h.x - wy * h.y));
-              out.y = om * (2.f * oc.y - (wx * h.y + wy * h.x));
+              out = jacobi2(om, d, oc, h);
               if (a.base) {
                 out.x += bq[r][j][i].x;
                 out.y += bq[r][j][i].y;
@@ -1018,7 +1010,7 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
   if (tid == 0 && dead) {
     for (int i = 0; i < min(NSTG, dead); ++i) {
       int gone = 0;
-      mbar_wait(full + 8 * i, (unsigned)((dead - 1 - i) / NSTG) & 1, gone, 1, a.err, a.polls);
+      mbar_wait(full + 8 * i, (unsigned)((dead - 1 - i) / NSTG) & 1, gone, 1, a);
     }
   }
   if constexpr (MODE == M_RESID) reduce_norm<RB>(a, reinterpret_cast<double*>(smem + SM::o_red), nrm2, rhs0, bid, nblk);
@@ -1053,7 +1045,7 @@ __device__ __forceinline__ void pml_body(const StencilCall<float>& a, unsigned c
                                          unsigned nblk) {
   using SM = PmlSmem<MODE>;
   constexpr int NSTG = SM::NSTG, PREF = SM::PREF;
-  constexpr bool J2 = SM::J2, OWN = SM::OWN, XC = FORM != 3, ZP = FORM == 2, TC = OPK == OPK_A;
+  constexpr bool J2 = SM::J2, OWN = SM::OWN, XC = FORM != 3, ZP = FORM == 2;
   const LevelView<float>& L = a.lv;
   const unsigned sb = (unsigned)__cvta_generic_to_shared(smem);
   float2* sEz = reinterpret_cast<float2*>(smem + SM::o_ez);
@@ -1063,23 +1055,13 @@ __device__ __forceinline__ void pml_body(const StencilCall<float>& a, unsigned c
   const int ty = tid / (tw / 2), tx = 2 * (tid - ty * (tw / 2));
   const long long plane = (long long)nx * ny;
   const long long xs = a.xstride > 0 ? a.xstride : L.N, ys = a.ystride > 0 ? a.ystride : L.N;
-  SegK K;
-  const int nq = a.tab.nseg * (TC ? L.nsub : 1);
-  K.s1 = a.tab.inv_ds * (float)kInv2Pi * (TC ? (float)L.nsub : 1.f);
-  K.hi = (float)nq;
-  K.sc = K.s1 / K.hi;
-  K.off = -0.5f / K.hi;
-  {
-    const int ns = a.tab.nseg + 1;
-    const float4* g = reinterpret_cast<const float4*>(L.mtab + (TC ? mt_off_S(ns) : kMtC * ns));
-    float4* t = reinterpret_cast<float4*>(smem + SM::o_tab);
-    for (int i = tid; i < 6 * (nq + 1); i += NT) t[i] = g[i];
-    if constexpr (ZP)
-      for (int i = tid; i < zb1 - zb0; i += NT) {
-        sEz[2 * i] = ldf2(L.eps[2][0] + zb0 + i);
-        sEz[2 * i + 1] = ldf2(L.eps[2][1] + zb0 + i);
-      }
-  }
+  const SegK K = tab_seg<OPK>(a);
+  load_table<OPK>(a, smem + SM::o_tab);
+  if constexpr (ZP)
+    for (int i = tid; i < zb1 - zb0; i += NT) {
+      sEz[2 * i] = ldf2(L.eps[2][0] + zb0 + i);
+      sEz[2 * i + 1] = ldf2(L.eps[2][1] + zb0 + i);
+    }
   // this thread's columns; threads past the tile or its bounds compute columns of
   // the grid that nobody stores
   const bool act0 = ty < th && x0 + tx <= rx1 && y0 + ty <= ry1, act1 = act0 && x0 + tx + 1 <= rx1;
@@ -1266,7 +1248,7 @@ __device__ __forceinline__ void pml_body(const StencilCall<float>& a, unsigned c
       n.k = add2(h[0][i], h[2][i]);
       const float kp1 = i ? kap.y : kap.x;
       float wt[8], a45[2];
-      core_weights<OPK, true>(K, tab, kp1, wt, a45);
+      row_weights<OPK, true>(K, tab, kp1, wt, a45);
       [[maybe_unused]] const float2 oc = w[i].c;  // the row's own value
       const float2 hv = row_value<OPK, true, ZP>(wt, kp1 * kp1, inv_l2, sigma, w[i], n, nA[i], nB[i], zp, ezp, ezm, a45[0], a45[1]);
       if (fin && (i ? act1 : act0)) {
@@ -1274,12 +1256,10 @@ __device__ __forceinline__ void pml_body(const StencilCall<float>& a, unsigned c
         if constexpr (OWN) {
           const float2 g = i ? make_float2(gq.z, gq.w) : make_float2(gq.x, gq.y);
           if constexpr (J2) {
-            // with y1 = omega D^-1 g and c = y1 / omega:
-            // y1 + omega D^-1 (g - H y1) = omega (2 c - omega D^-1 H c)
             const float2 d = lds64(r0 + sop + SM::o_d + 8 * (pw + 1 + i));
-            const float wx = om * d.x, wy = om * d.y;
-            out.x = om * (2.f * oc.x - (wx * hv.x - wy * hv.y)) + g.x;
-            out.y = om * (2.f * oc.y - (wx * hv.y + wy * hv.x)) + g.y;
+            out = jacobi2(om, d, oc, hv);
+            out.x += g.x;
+            out.y += g.y;
           } else {
             out = make_float2(g.x - hv.x, g.y - hv.y);
             if constexpr (MODE == M_RESID) {
@@ -1306,8 +1286,10 @@ __device__ __forceinline__ void pml_body(const StencilCall<float>& a, unsigned c
   if constexpr (MODE == M_RESID) reduce_norm<1>(a, reinterpret_cast<double*>(smem + SM::o_red), &nrm2, rhs, bid, nblk);
 }
 
+// (the residual of two right-hand sides spills 100 bytes at four blocks per SM: 153^3
+// A 92.9 us, 85.4 at three)
 template <int MODE, int OPK, int NPY, int RB>
-__global__ void __launch_bounds__(NT, RB == 2 ? 4 : 3) k_march(const __grid_constant__ StencilCall<float> a, const __grid_constant__ Plan pl,
+__global__ void __launch_bounds__(NT, RB == 2 && MODE != M_RESID ? 4 : 3) k_march(const __grid_constant__ StencilCall<float> a, const __grid_constant__ Plan pl,
                const __grid_constant__ Maps mp) {
   extern __shared__ __align__(128) unsigned char fsm[];
   const unsigned nb = (unsigned)pl.items;
@@ -1348,12 +1330,12 @@ __global__ void __launch_bounds__(NT, RB == 2 ? 4 : 3) k_march(const __grid_cons
   }
 }
 
-// Dynamic shared memory of a launch: parts of the table the bodies copy; the core
-// by TMA (rows) or element by element.
+// Dynamic shared memory of a launch: rows of its table without the clamp; the core
+// by TMA (tma) or element by element.
 template <int MODE, int OPK, int NPY, int RB>
-constexpr size_t march_smem(int parts, bool rows) {
-  const size_t tab = (size_t)96 * (parts + 1);
-  const size_t core = rows ? CoreSmem<MODE, NPY, RB>::o_tab + tab : Smem<MODE, CoreT<NPY>, RB>::bytes;
+constexpr size_t march_smem(int rows, bool tma) {
+  const size_t tab = (size_t)4 * kTabRow<OPK> * (rows + 1);
+  const size_t core = (tma ? (size_t)CoreSmem<MODE, NPY, RB>::o_tab : Smem<MODE, CoreT<NPY>, RB>::o_tab) + tab;
   return OPK == OPK_Q ? core : std::max(core, PmlSmem<MODE>::o_tab + tab);
 }
 

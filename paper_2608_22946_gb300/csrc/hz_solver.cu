@@ -456,19 +456,17 @@ void build_march_tables(const std::vector<double>& coef, const double* rows, int
   const int ns = K;
   out.assign((size_t)march::mt_size(ns), 0.f);
   const double inv_l2 = 1.0 / (ell * ell);
-  const size_t oF = (size_t)march::kMtC * ns, oQ = oF + (size_t)march::kMtF * ns;
+  const size_t oF = (size_t)march::mt_off_F(ns);
   for (int k = 0; k < ns; ++k) {
     const MarchFns F = march_fns(coef, rows, K, ds, k);
-    for (int m = 0; m < 4; ++m) {
-      for (int j = 0; j < 6; ++j) out[(size_t)k * march::kMtC + 4 * j + m] = (float)(inv_l2 * F.Cm[m][j]);
-      for (int j = 0; j < 4; ++j) {
-        out[oF + (size_t)k * march::kMtF + 6 * j + 2 + m] = (float)F.Mm[m][j];
-        out[oQ + (size_t)k * march::kMtQ + 4 * j + m] = (float)F.Qm[m][j];
-      }
-    }
     for (int j = 0; j < 4; ++j) {
-      out[oF + (size_t)k * march::kMtF + 6 * j] = (float)F.a4[j];
-      out[oF + (size_t)k * march::kMtF + 6 * j + 1] = (float)F.a5[j];
+      float* f = &out[oF + (size_t)k * march::kMtF + 6 * j];
+      f[0] = (float)(F.a4[j] - (j == 0 ? march::kA4Off : 0.0));
+      f[1] = (float)(F.a5[j] - (j == 0 ? march::kA5Off : 0.0));
+      for (int m = 0; m < 4; ++m) {
+        f[2 + m] = (float)F.Mm[m][j];
+        out[(size_t)k * march::kMtQ + 4 * j + m] = (float)F.Qm[m][j];
+      }
     }
     for (int b = 0; b < (k < K - 1 ? nsub : 1); ++b)
       for (int m = 0; m < 6; ++m) {

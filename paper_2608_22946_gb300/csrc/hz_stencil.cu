@@ -143,7 +143,7 @@ __device__ __forceinline__ void adj_tile(const StencilCall<R>& a, unsigned char*
       cx<R> v = xv[j];
       if constexpr (MODE == M_J2) v = cjmul(dv[j], v);  // y1 / omega = D^-H g
       R u, C[4];
-      const int seg = seg_of(kv[j], ns, ds, inv_ds, u);
+      const int seg = seg_exact(kv[j], ns, ds, inv_ds, u);
       if constexpr (Q) {
         horner_pm<R, 4, 3>(sT + seg * kCtQ, u, C);
 #pragma unroll
@@ -184,8 +184,9 @@ __device__ __forceinline__ void adj_tile(const StencilCall<R>& a, unsigned char*
     const cx<R>* F = sF + (size_t)buf * kAdjF * PLANE + lc;
     auto face = [&](const cx<R>* f) { return (f[-1] + f[1]) + (f[-PW] + f[PW]); };
     auto corner = [&](const cx<R>* f) { return (f[-PW - 1] + f[-PW + 1]) + (f[PW - 1] + f[PW + 1]); };
-    cx<R> p0 = F[0] + face(F + PLANE) + corner(F + 2 * PLANE);
-    cx<R> p1 = F[PLANE] + face(F + 2 * PLANE) + corner(F + 3 * PLANE);
+    // (the small terms first: one rounding at the size of the large one)
+    cx<R> p0 = (corner(F + 2 * PLANE) + face(F + PLANE)) + F[0];
+    cx<R> p1 = (corner(F + 3 * PLANE) + face(F + 2 * PLANE)) + F[PLANE];
     cx<R> pm = p1, pp = p1;
     if constexpr (GEN) {
       const cx<R>*v0 = F + 4 * PLANE, *v1 = F + 5 * PLANE, *v2 = F + 6 * PLANE;
