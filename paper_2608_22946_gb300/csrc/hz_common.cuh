@@ -144,6 +144,7 @@ struct LevelView {
   R inv_ell2;                     // 1 / ell^2
   int zblock;                     // planes per CTA of the forward stencil (0: heuristic)
   int zblock_f;                   // the same for the PML-frame launch (0: as zblock)
+  int zb_march, zb_march_f;       // the same two for the single-precision march
 };
 
 // ----------------------------------------------------------------------------

@@ -647,22 +647,53 @@ __global__ void __launch_bounds__(TileS::NTH) k_fwd_small(StencilCall<R> a, int 
 // ----------------------------------------------------------------------------
 // launcher
 // ----------------------------------------------------------------------------
-static int choose_zblock(int nx, int ny, int nz, int nrhs) {
-  if ((long long)nx * ny * nz <= kSmallNodes) return kMinZblock;
-  long long tiles = (long long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY) * nrhs;
-  // aim for about 4 waves of 2 CTAs on 152 SMs, with at least 4 planes per CTA
-  long long want = 152LL * 2 * 4;
-  long long nzb = (want + tiles - 1) / tiles;
-  int zb = (int)((nz + nzb - 1) / nzb);
-  if (zb < 4) zb = 4;
-  if (zb > 64) zb = 64;
-  return zb;
-}
-
 // Grids of at least this many nodes split interior and PML tiles into two
 // launches (each kernel then carries only its own path's registers); smaller
 // grids, where launch latency dominates, use one launch choosing per tile.
 constexpr long long kSplitNodes = 1LL << 20;
+
+// Planes per block where no tuned value applies.
+static int choose_zblock(bool single, int nx, int ny, int nz, int nrhs) {
+  const long long n = (long long)nx * ny * nz;
+  auto per_block = [&](long long nzb, int lo, int hi) {  // nzb z-blocks, lo .. hi planes each
+    nzb = std::max(nzb, 1LL);
+    return (int)std::min<long long>(std::max<long long>((nz + nzb - 1) / nzb, lo), hi);
+  };
+  if (n <= kSmallNodes) {
+    const long long tiles = (long long)((nx + 7) / 8) * ((ny + 7) / 8) * nrhs;  // 8 x 8 tiles
+    if (single) {
+      // two planes per block while blocks are what the GPU lacks, more as right-hand
+      // sides supply them (the two halo planes are loaded for every block): J_2 on 41^3
+      // with 1, 2, 4, 8 right-hand sides 5.1, 9.0, 13.4, 22.3 us at two planes; 5.3, 6.9,
+      // 10.3, 16.6 at 2, 3, 6, 12
+      return (int)std::min<long long>(std::max<long long>(n * nrhs / 40000, 2), 12);
+    }
+    // FP64 rate: an SM works through its blocks' planes one after the other once it has
+    // two of them, and a plane takes no less than two blocks' time (49^3 J_2: 74 us at
+    // two planes, 65 at three; 25^3 with four right-hand sides 72 at two, 55 at four)
+    int best = kMinZblock;
+    double cost = 1e30;
+    for (int zb = kMinZblock; zb <= 12; ++zb) {
+      const long long blocks = tiles * ((nz + zb - 1) / zb);
+      const double c = (zb + 2) * std::max(2.2, (double)((blocks + 151) / 152));
+      if (c < cost - 1e-9) {
+        cost = c;
+        best = zb;
+      }
+    }
+    return best;
+  }
+  if (single && n < kSplitNodes) {
+    // one wave of two to three blocks of 16 x 16 columns per SM: every z-block loads two
+    // planes more than it writes (97^3 J_2 25.1 us at 5 planes, 20.9 at 16; 81^3 17.9 at
+    // 4, 14.7 at 10)
+    return per_block(340 / ((long long)((nx + 15) / 16) * ((ny + 15) / 16) * nrhs), 4, 34);
+  }
+  // about 4 waves of 2 blocks on 152 SMs, at least 4 planes per block
+  const long long tiles = (long long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY) * nrhs;
+  return per_block((152LL * 2 * 4 + tiles - 1) / tiles, 4, 64);
+}
+
 
 static int cdiv_i(int a, int b) { return a > 0 ? (a + b - 1) / b : 0; }
 
@@ -727,7 +758,7 @@ static FwdPlan plan_layout(int nx, int ny, int nz, const int* plo, const int* ph
 
 template <class R>
 static FwdPlan plan_fwd(const LevelView<R>& L, int nrhs, int op) {
-  const int zb = L.zblock > 0 ? L.zblock : choose_zblock(L.nx, L.ny, L.nz, nrhs);
+  const int zb = L.zblock > 0 ? L.zblock : choose_zblock(sizeof(R) == sizeof(float), L.nx, L.ny, L.nz, nrhs);
   return plan_layout(L.nx, L.ny, L.nz, L.plain_lo, L.plain_hi, op, zb, L.zblock_f);
 }
 
@@ -784,9 +815,9 @@ static void launch_fwd_t(const StencilCall<R>& c, cudaStream_t s) {
 
 // Blocks per right-hand side of a forward stencil launch on this grid (the
 // size of the per-block partial-sum array its reductions need).
-long long gather_blocks_per_rhs(int nx, int ny, int nz, const int* plain_lo, const int* plain_hi, int nrhs,
-                                int zblock, int zblock_f) {
-  const int zb = zblock > 0 ? zblock : choose_zblock(nx, ny, nz, nrhs);
+long long gather_blocks_per_rhs(bool single, int nx, int ny, int nz, const int* plain_lo, const int* plain_hi,
+                                int nrhs, int zblock, int zblock_f) {
+  const int zb = zblock > 0 ? zblock : choose_zblock(single, nx, ny, nz, nrhs);
   const FwdPlan p = plan_layout(nx, ny, nz, plain_lo, plain_hi, OP_AB, zb, zblock_f);
   return p.blocks();
 }
@@ -799,9 +830,9 @@ long long gather_blocks_per_rhs(int nx, int ny, int nz, const int* plain_lo, con
 // axes, form 1 y, form 3 x), a block id out of range or repeated.  counts
 // (nx * ny * nz bytes, or null) receives how often each node of right-hand
 // side 0 is written, saturating at 255.
-long long replay_gather_layout(int nx, int ny, int nz, const int* plo, const int* phi, int op, int nrhs,
+long long replay_gather_layout(bool single, int nx, int ny, int nz, const int* plo, const int* phi, int op, int nrhs,
                                int zblock, int zblock_f, unsigned char* counts, long long* blocks) {
-  const int zb = zblock > 0 ? zblock : choose_zblock(nx, ny, nz, nrhs);
+  const int zb = zblock > 0 ? zblock : choose_zblock(single, nx, ny, nz, nrhs);
   const FwdPlan p = plan_layout(nx, ny, nz, plo, phi, op, zb, zblock_f);
   const long long nblk = p.blocks();
   if (blocks) *blocks = nblk;

@@ -114,28 +114,50 @@ constexpr long long kSmallNodes = 1LL << 17;
 
 namespace march {
 // forward stencil in single precision, every level (hz_march.cuh)
+// The core's planes come by TMA where rows of two pair up to 16 bytes and the core's
+// halo lies inside the grid (hz_march.cuh), else element by element.
+inline bool core_by_tma(int nx, int ny, int nz, const int* plo, const int* phi) {
+  return nx % 2 && ny % 2 && plo[0] > 1 && phi[0] < nx - 3 && plo[1] > 1 && phi[1] < ny - 2 && plo[2] > 1 &&
+         phi[2] + 1 < nz - 1;
+}
 // Small grids take the gather-form kernels of hz_fwd_gather.cu, on every level:
 // their marches are a few planes long, and the longer prologue (tables, the
 // copies' latency) and larger code of the march cost more than its steady state
-// gains, the more so the more the mode stages.  In a graph, us, gather / march:
-//   apply B     39^3 4.3 / 5.6, 73^3 8.2 / 8.7, 77^3 10.0 / 10.0, 89^3 13.1 / 13.1
-//               (A 13.1 / 12.1), 97^3 16.2 / 16.1, 113^3 21.7 / 20.6, 129^3 31 / 25.7
-//   residual    97^3 25.6 / 27.9, 113^3 38.2 / 34.8; two right-hand sides 41.1 /
-//               49.3 and 61 / 53.6
-//   J_2         97^3 20.0 / 24.8, 113^3 28.5 / 30.8, 129^3 41.6 / 37.8; two
-//               right-hand sides 97^3 37.4 / 38.9, 113^3 51 / 47.2
-inline bool takes(int mode, int nx, int ny, int nz, int nrhs) {
-  const long long n = (long long)nx * ny * nz;
+// gains, the more so the more the mode stages.  The march shares a block's weights
+// between two right-hand sides, so there the lines lie lower; more than two move them
+// no further (77^3 with 8, B: J_2 57 / 74).  The fine level's gather rows cost more
+// (combined quintics) than the coarse levels', B's march rows more than A's.  In a
+// graph, each at its best z-block, us, gather / march:
+//   apply A     77^3 10.1 / 11.0, 81^3 12.1 / 10.7; two right-hand sides 20.8 / 16.6
+//   apply B     97^3 16.7 / 16.6, 105^3 17.6 / 17.8, 113^3 22.9 / 20.5; two 81^3 20.0 /
+//               18.8, 89^3 21.6 / 23.3, 97^3 29.5 / 27.5
+//   residual    97^3 25.6 / 27.9, 113^3 38.2 / 34.8; two 41.1 / 49.3 and 61 / 53.6
+//   J_2 A       97^3 20.9 / 23.6, 105^3 28.3 / 27.1, 113^3 30.5 / 27.9; two 97^3 37.5 /
+//               38.6, 105^3 46.7 / 43.1
+//   J_2 B       113^3 30.9 / 31.4, 129^3 38.5 / 37.7; two 105^3 39.3 / 47, 113^3 50.4 /
+//               50.9, 121^3 57 / 54
+// and J_2 where the core comes element by element (no PML), which passes each plane
+// through shared memory twice: 121^3 24.1 / 21.6, 141^3 34.8 / 38.9, 201^3 84.9 / 90.0;
+// two 121^3 39.0 / 38.8, 141^3 60.7 / 75.4, 201^3 158 / 192; four on 289^2 x 269 790 / 727.
+inline bool takes(int mode, bool shifted, int nx, int ny, int nz, int nrhs, const int* plo, const int* phi) {
+  const long long n = (long long)nx * ny * nz, n2 = n * (nrhs > 1 ? 2 : 1);
   if (mode == M_RESID) return n >= 1LL << 20;
-  if (mode == M_J2) return n * (nrhs > 1 ? 2 : 1) >= 1LL << 21;
-  return n >= 1LL << 19;
+  if (mode == M_J2) {
+    if (!core_by_tma(nx, ny, nz, plo, phi) && n >= 1LL << 21 && n < 1LL << 24) return false;
+    return shifted ? n2 >= 5LL << 19 : n >= 1LL << 20;
+  }
+  return shifted ? n2 >= 1LL << 20 : n >= 1LL << 19;
+}
+inline bool takes(const LevelView<float>& L, int mode, bool shifted, int nrhs) {
+  return takes(mode, shifted, L.nx, L.ny, L.nz, nrhs, L.plain_lo, L.plain_hi);
 }
 void launch(const StencilCall<float>& c, int mode, int opk, cudaStream_t s);
 void init_attrs();
 // Tiles of the PML strips of a grid (LevelView::strip); searched once per level.
 void strips(int nx, int ny, const int* plo, const int* phi, int* strip);
+// Blocks per right-hand side of a march at these z-blocks (0: its own).
 long long blocks_per_rhs(int nx, int ny, int nz, const int* plain_lo, const int* plain_hi, int nrhs, int zblock,
-                         int zblock_f, const int* strip = nullptr);
+                         int zblock_f, const int* strip);
 long long replay_layout(int nx, int ny, int nz, const int* plo, const int* phi, int op, int nrhs, int zblock,
                         int zblock_f);
 }  // namespace march
@@ -145,10 +167,10 @@ namespace gather {
 // single precision (hz_fwd_gather.cu)
 template <class R>
 void launch_fwd_gather(const StencilCall<R>& c, int mode, int op, cudaStream_t s);
-long long gather_blocks_per_rhs(int nx, int ny, int nz, const int* plain_lo, const int* plain_hi, int nrhs,
-                                int zblock, int zblock_f);
-long long replay_gather_layout(int nx, int ny, int nz, const int* plo, const int* phi, int op, int nrhs, int zblock,
-                               int zblock_f, unsigned char* counts, long long* blocks);
+long long gather_blocks_per_rhs(bool single, int nx, int ny, int nz, const int* plain_lo, const int* plain_hi,
+                                int nrhs, int zblock, int zblock_f);
+long long replay_gather_layout(bool single, int nx, int ny, int nz, const int* plo, const int* phi, int op, int nrhs,
+                               int zblock, int zblock_f, unsigned char* counts, long long* blocks);
 // The bottom solve C_4h (s-step CA-GMRES with kBottomSteps steps, two-sweep
 // Jacobi maps of B_4h) as one persistent cooperative kernel.
 constexpr int kBottomSteps = 4;

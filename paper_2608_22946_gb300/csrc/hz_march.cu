@@ -57,6 +57,20 @@ static Plan make_plan(int nx, int ny, const int* plo, const int* phi, const int*
   return p;
 }
 
+// Right-hand sides per block (they share its coefficients): two, or one with two
+// rows of columns per thread; a thread carries four columns' state either way.
+static int pick_rb(int nrhs) { return nrhs % 2 == 0 ? 2 : 1; }
+
+// Planes per block where no tuned value applies: about two waves of three core blocks
+// per SM, 8 to 34 planes (two are loaded on top of them: 105^3 A_h 19.8 us at 4, 17.0
+// at 12; B with two right-hand sides on 81^3 24.1 at 4, 18.8 at 8).
+static int choose_zb(int nx, int ny, int nz, int nrhs) {
+  const int rb = pick_rb(nrhs);
+  const long long tiles = (long long)cdiv_i(nx, 64) * cdiv_i(ny, rb == 2 ? 4 : 8) * (nrhs / rb);
+  const long long nzb = std::max(1LL, 152 * 3 * 2 / tiles);
+  return (int)std::min<long long>(std::max<long long>((nz + nzb - 1) / nzb, 8), 34);
+}
+
 // Tensor map of a field of `rows` rows of nx complex64 values as lines of two
 // rows (CoreSmem's comment); `lines` lines of 68 values per copy.
 static bool field_map(CUtensorMap* m, const void* base, int nx, long long rows, int lines) {
@@ -82,11 +96,11 @@ static bool field_map(CUtensorMap* m, const void* base, int nx, long long rows, 
                 CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int MODE, int OPK, int NPY, int RB>
+template <int MODE, int OPK, int NPY, int RB, int MB>
 static void launch_t(const StencilCall<float>& c, cudaStream_t s) {
   const LevelView<float>& L = c.lv;
-  const int zb = L.zblock > 0 ? L.zblock : choose_zblock(L.nx, L.ny, L.nz, c.nrhs);
-  Plan p = make_plan(L.nx, L.ny, L.plain_lo, L.plain_hi, L.strip, OPK != OPK_Q, zb, L.zblock_f, NPY, c.zr0,
+  const int zb = L.zb_march > 0 ? L.zb_march : choose_zb(L.nx, L.ny, L.nz, c.nrhs);
+  Plan p = make_plan(L.nx, L.ny, L.plain_lo, L.plain_hi, L.strip, OPK != OPK_Q, zb, L.zb_march_f, NPY, c.zr0,
                            c.zr1 > 0 ? c.zr1 : L.nz);
   count_launch();
   // (two right-hand sides per block: the second one's rows must start on the other 8-byte half)
@@ -101,27 +115,37 @@ static void launch_t(const StencilCall<float>& c, cudaStream_t s) {
     if (MODE == M_J2) p.rows = p.rows && field_map(&mp.d, c.dinv, L.nx, L.N / L.nx, 2 * NPY + 1);
   }
   const unsigned blocks = (unsigned)p.nfr * c.nrhs + (unsigned)(p.items - p.nfr) * (c.nrhs / RB);
-  k_march<MODE, OPK, NPY, RB><<<blocks, NT, march_smem<MODE, OPK, NPY, RB>(c.tab.nseg * (OPK == OPK_A ? L.nsub : 1), p.rows), s>>>(c, p, mp);
+  k_march<MODE, OPK, NPY, RB, MB><<<blocks, NT, march_smem<MODE, OPK, NPY, RB>(c.tab.nseg * (OPK == OPK_A ? L.nsub : 1), p.rows), s>>>(c, p, mp);
 }
-
-// Right-hand sides per block (they share its coefficients): two, or one with two
-// rows of columns per thread; a thread carries four columns' state either way.
-static int pick_rb(int nrhs) { return nrhs % 2 == 0 ? 2 : 1; }
 
 template <int MODE, int OPK>
 void launch_mode(const StencilCall<float>& c, cudaStream_t s) {
-  if (pick_rb(c.nrhs) == 2) launch_t<MODE, OPK, 1, 2>(c, s);
-  else launch_t<MODE, OPK, 2, 1>(c, s);
+  // residual of two, A, us at three / four blocks per SM: 119^3 62 / 56, 137 x 125 x 113
+  // 68 / 64, 153^3 88 / 122, 289^3 347 / 418
+  if (pick_rb(c.nrhs) == 2) {
+    if constexpr (MODE == M_RESID) {
+      if (c.lv.N >= 5LL << 19) {
+        launch_t<MODE, OPK, 1, 2, 3>(c, s);
+        return;
+      }
+    }
+    launch_t<MODE, OPK, 1, 2, 4>(c, s);
+  } else {
+    launch_t<MODE, OPK, 2, 1, 3>(c, s);
+  }
 }
 
+template <int MODE, int OPK, int NPY, int RB, int MB>
+static void set_attr() {
+  cudaFuncSetAttribute(k_march<MODE, OPK, NPY, RB, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)std::max(march_smem<MODE, OPK, NPY, RB>(kMaxParts, true),
+                                     march_smem<MODE, OPK, NPY, RB>(kMaxParts, false)));
+}
 template <int MODE, int OPK>
 void mode_attrs() {
-  cudaFuncSetAttribute(k_march<MODE, OPK, 1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)std::max(march_smem<MODE, OPK, 1, 2>(kMaxParts, true),
-                                     march_smem<MODE, OPK, 1, 2>(kMaxParts, false)));
-  cudaFuncSetAttribute(k_march<MODE, OPK, 2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)std::max(march_smem<MODE, OPK, 2, 1>(kMaxParts, true),
-                                     march_smem<MODE, OPK, 2, 1>(kMaxParts, false)));
+  set_attr<MODE, OPK, 1, 2, 4>();
+  if constexpr (MODE == M_RESID) set_attr<MODE, OPK, 1, 2, 3>();
+  set_attr<MODE, OPK, 2, 1, 3>();
 }
 
 #define HZ_MARCH_INST(KW, MODE, OPK)                                                  \
@@ -199,7 +223,7 @@ void strips(int nx, int ny, const int* plo, const int* phi, int* strip) {
 static Plan plan_of(int nx, int ny, int nz, const int* plo, const int* phi, bool ab, int nrhs, int zblock,
                     int zblock_f, const int* strip, int& npy) {
   npy = pick_rb(nrhs) == 2 ? 1 : 2;
-  const int zb = zblock > 0 ? zblock : choose_zblock(nx, ny, nz, nrhs);
+  const int zb = zblock > 0 ? zblock : choose_zb(nx, ny, nz, nrhs);
   int own[4];
   if (!strip) {
     strips(nx, ny, plo, phi, own);
@@ -210,7 +234,6 @@ static Plan plan_of(int nx, int ny, int nz, const int* plo, const int* phi, bool
 
 long long blocks_per_rhs(int nx, int ny, int nz, const int* plo, const int* phi, int nrhs, int zblock, int zblock_f,
                          const int* strip) {
-  if (!takes(M_RESID, nx, ny, nz, nrhs)) return gather::gather_blocks_per_rhs(nx, ny, nz, plo, phi, nrhs, zblock, zblock_f);
   int npy;
   return plan_of(nx, ny, nz, plo, phi, true, nrhs, zblock, zblock_f, strip, npy).items;
 }

@@ -184,15 +184,18 @@ __device__ __forceinline__ float2 row_value(const float* w, float k2, float inv_
     N2 = add2(s.p2, n.e);
   }
   const float2 N3 = add2(s.p3, n.k);
-  // Terms are added smallest first (PML corrections, corners inwards): only the last
-  // addition then rounds at the size of the centre's term.
+  // Terms are added smallest first (corners inwards, PML corrections before the faces):
+  // only the last addition then rounds at the size of the centre's term.
+  float2 h = make_float2(w[3] * N3.x, w[3] * N3.y);
+  rfma(h, w[2], N2);
+  // (B scales its rows by ell^-2 at the end: its corrections wait in a sum of their own)
   [[maybe_unused]] float2 cor = make_float2(0.f, 0.f);
   if constexpr (CORR) {
     const float q5 = 0.25f * a5, qb = fmaf(-0.25f, a4 + a5, 0.25f);
-    const float2 A1 = add2(s.BA, nA), B1 = add2(s.Bm, nB);
-    cor = make_float2(qb * B1.x, qb * B1.y);
-    rfma(cor, q5, A1);
-    rfma(cor, a4, s.A);
+    float2& t0 = OPK == OPK_B ? cor : h;
+    rfma(t0, qb, add2(s.Bm, nB));
+    rfma(t0, q5, add2(s.BA, nA));
+    rfma(t0, a4, s.A);
     s.BA = add2(nB, s.A);
     s.Bm = s.B;
     s.A = nA;
@@ -203,23 +206,15 @@ __device__ __forceinline__ float2 row_value(const float* w, float k2, float inv_
         rfma(t, qb, sub2(n.k, s.k));
         rfma(t, q5, sub2(n.e, s.e));
         rfma(t, a4, sub2(n.c, s.c));
-        cfma2(cor, ezp, t);
+        cfma2(t0, ezp, t);
         t = make_float2(0.f, 0.f);
         rfma(t, qb, sub2(s.p3, s.k));
         rfma(t, q5, sub2(s.p2, s.e));
         rfma(t, a4, sub2(s.p1, s.c));
-        cfma2(cor, ezm, t);
+        cfma2(t0, ezm, t);
       }
     }
   }
-  float2 h;
-  if constexpr (OPK != OPK_B && CORR) {
-    h = cor;
-    rfma(h, w[3], N3);
-  } else {
-    h = make_float2(w[3] * N3.x, w[3] * N3.y);
-  }
-  rfma(h, w[2], N2);
   rfma(h, w[1], N1);
   rfma(h, w[0], s.c);
   if constexpr (OPK == OPK_B) {
@@ -1286,10 +1281,11 @@ __device__ __forceinline__ void pml_body(const StencilCall<float>& a, unsigned c
   if constexpr (MODE == M_RESID) reduce_norm<1>(a, reinterpret_cast<double*>(smem + SM::o_red), &nrm2, rhs, bid, nblk);
 }
 
-// (the residual of two right-hand sides spills 100 bytes at four blocks per SM: 153^3
-// A 92.9 us, 85.4 at three)
-template <int MODE, int OPK, int NPY, int RB>
-__global__ void __launch_bounds__(NT, RB == 2 && MODE != M_RESID ? 4 : 3) k_march(const __grid_constant__ StencilCall<float> a, const __grid_constant__ Plan pl,
+// MB: blocks per SM.  Three, or four where a block carries one row of columns for two
+// right-hand sides; the residual of two spills 100 bytes at four, which grids that fill
+// the GPU three times over pay for (launch_mode).
+template <int MODE, int OPK, int NPY, int RB, int MB>
+__global__ void __launch_bounds__(NT, MB) k_march(const __grid_constant__ StencilCall<float> a, const __grid_constant__ Plan pl,
                const __grid_constant__ Maps mp) {
   extern __shared__ __align__(128) unsigned char fsm[];
   const unsigned nb = (unsigned)pl.items;

@@ -107,6 +107,7 @@ struct Level {
   cx<double>* dinv_d[2] = {};
   int zblock = 0;    // forward-stencil planes per thread block (autotuned; 0: heuristic)
   int zblock_f = 0;  // the same for the PML-frame launch (0: as zblock)
+  int zfam = 0;      // kernels they were timed on (ZFam)
 };
 
 template <class R>
@@ -165,7 +166,7 @@ struct hz_handle {
   double *s_nrm = nullptr, *s_root = nullptr, *s_inv = nullptr;
   std::map<std::tuple<int, int, int, const void*, void*>, std::pair<cudaGraphExec_t, unsigned long long>> graphs;
   double t_setup = 0;
-  bool tuned_c64 = false;  // z-blocks were timed in single precision
+  bool tuned_single = false;  // precision the z-blocks were timed in
   bool use_graphs = true;
   // the bottom solve C_4h as one persistent cooperative kernel (forward, m_4h = 4,
   // two Jacobi sweeps; opt-in through HZ_PERSISTENT=1 at creation); its
@@ -482,6 +483,14 @@ void build_march_tables(const std::vector<double>& coef, const double* rows, int
   }
 }
 
+// The three forward kernel designs.  A tuned z-block serves the one and the precision
+// it was timed in, the others take their own rules.
+enum ZFam { Z_NONE = 0, Z_ACCUM, Z_GATHER, Z_MARCH };
+// the design of the calls that do not march
+int plain_fam(bool single, int L, const Level& lv) {
+  return !single && L == 0 && lv.N > kSmallNodes ? Z_ACCUM : Z_GATHER;
+}
+
 template <class R>
 LevelView<R> view(hz_handle* H, int L) {
   const Level& lv = H->lev[L];
@@ -505,10 +514,12 @@ LevelView<R> view(hz_handle* H, int L) {
   v.nsub = H->nsub;
   for (int i = 0; i < 4; ++i) v.strip[i] = lv.strip[i];
   v.inv_ell2 = (R)(1.0 / (lv.ell * lv.ell));
-  v.zblock = lv.zblock;
-  v.zblock_f = lv.zblock_f;
-  // z-blocks tuned on the complex64 kernels say nothing about the FP64-bound ones
-  if (sizeof(R) == sizeof(double) && H->tuned_c64) v.zblock = v.zblock_f = 0;
+  const bool tuned = H->tuned_single == (sizeof(R) == sizeof(float)), march = tuned && lv.zfam == Z_MARCH;
+  const bool same = tuned && lv.zfam == plain_fam(sizeof(R) == sizeof(float), L, lv);
+  v.zblock = same ? lv.zblock : 0;
+  v.zblock_f = same ? lv.zblock_f : 0;
+  v.zb_march = march ? lv.zblock : 0;
+  v.zb_march_f = march ? lv.zblock_f : 0;
   return v;
 }
 template <class R>
@@ -945,9 +956,10 @@ long long resid_blocks(const Level& lv, int level, int nrhs, bool adjoint, int z
                  : stencil_blocks_per_rhs(level, lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nrhs, zblock, zblock_f);
 }
 
-long long fwd_blocks_c64(const Level& lv, int nrhs) {
-  return march::blocks_per_rhs(lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nrhs, lv.zblock, lv.zblock_f,
-                                lv.strip);
+long long fwd_blocks_c64(const LevelView<float>& v, int nrhs) {
+  return march::takes(v, M_RESID, false, nrhs)
+             ? march::blocks_per_rhs(v.nx, v.ny, v.nz, v.plain_lo, v.plain_hi, nrhs, v.zb_march, v.zb_march_f, v.strip)
+             : gather::gather_blocks_per_rhs(true, v.nx, v.ny, v.nz, v.plain_lo, v.plain_hi, nrhs, v.zblock, v.zblock_f);
 }
 
 // Per-block partial sums: the vector reductions use at most 1216 x 56, a fused
@@ -960,6 +972,8 @@ size_t red_partial_size(const Level* lev, int nrhs) {
                                                1, kMinZblock, kMinZblock);
     const long long a = adj_blocks_per_rhs(lev[L].nx, lev[L].ny, lev[L].nz, 1, kMinZblock);
     m = std::max(m, (size_t)std::max(f, a));
+    m = std::max(m, (size_t)gather::gather_blocks_per_rhs(true, lev[L].nx, lev[L].ny, lev[L].nz, lev[L].plain_lo,
+                                                          lev[L].plain_hi, 1, kMinZblock, kMinZblock));
     for (int r = 1; r <= 2; ++r)  // (one and two right-hand sides per block tile differently)
       m = std::max(m, (size_t)march::blocks_per_rhs(lev[L].nx, lev[L].ny, lev[L].nz, lev[L].plain_lo, lev[L].plain_hi,
                                                     r, kMinZblock, kMinZblock, lev[L].strip));
@@ -1056,6 +1070,17 @@ template <class R>
 void autotune_zblocks(hz_handle* H) {
   Work<R>& W = Sel<R>::w(H);
   const int nr = H->max_nrhs;
+  // the launch each level runs most: the A_h apply on the fine level, the
+  // two-sweep Jacobi map of the shifted operator on the coarse levels
+  // (the V-cycle and the bottom solve)
+  auto tuned_mode = [](int L) { return L == 0 ? M_APPLY : M_J2; };
+  H->tuned_single = sizeof(R) == sizeof(float);
+  for (int L = 0; L < 3; ++L) {
+    Level& lv = H->lev[L];
+    const bool march = sizeof(R) == sizeof(float) && march::takes(tuned_mode(L), L > 0, lv.nx, lv.ny, lv.nz, nr,
+                                                                  lv.plain_lo, lv.plain_hi);
+    lv.zfam = march ? Z_MARCH : plain_fam(sizeof(R) == sizeof(float), L, lv);
+  }
   TuneKey key{};
   HZ_CK(cudaGetDevice(&key.dev));
   key.prec = (int)sizeof(R);
@@ -1086,10 +1111,7 @@ void autotune_zblocks(hz_handle* H) {
     const long long n = lv.N * nr;
     launch_zero<R>(src[L], n, H->st);
     HZ_LAUNCHED();
-    // the launch each level runs most: the A_h apply on the fine level, the
-    // two-sweep Jacobi map of the shifted operator on the coarse levels
-    // (the V-cycle and the bottom solve)
-    const int mode = L == 0 ? M_APPLY : M_J2;
+    const int mode = tuned_mode(L);
     auto time_apply = [&]() {
       StencilCall<R> c = call<R>(H, L, L > 0, nr);
       c.x = src[L];
@@ -1113,13 +1135,16 @@ void autotune_zblocks(hz_handle* H) {
       }
       return ms;
     };
-    const bool split =
-        sizeof(R) == sizeof(float)
-            ? march::blocks_per_rhs(lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr, kMinZblock, 64, lv.strip) !=
-                  march::blocks_per_rhs(lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr, kMinZblock, kMinZblock,
-                                        lv.strip)
-            : stencil_blocks_per_rhs(L, lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr, kMinZblock, 64) !=
-        stencil_blocks_per_rhs(L, lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr, kMinZblock, kMinZblock);
+    // does the launch have PML-frame blocks with a z-block of their own?
+    auto blocks = [&](int zbf) {
+      return lv.zfam == Z_MARCH    ? march::blocks_per_rhs(lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr, kMinZblock,
+                                                           zbf, lv.strip)
+             : lv.zfam == Z_GATHER ? gather::gather_blocks_per_rhs(sizeof(R) == sizeof(float), lv.nx, lv.ny, lv.nz,
+                                                                   lv.plain_lo, lv.plain_hi, nr, kMinZblock, zbf)
+                                   : stencil_blocks_per_rhs(L, lv.nx, lv.ny, lv.nz, lv.plain_lo, lv.plain_hi, nr,
+                                                            kMinZblock, zbf);
+    };
+    const bool split = blocks(64) != blocks(kMinZblock);
     for (int pass = 0; pass < (split ? 2 : 1); ++pass) {
       float best_t = 1e30f;
       int best = 0;
@@ -1858,7 +1883,6 @@ hz_status hz_create(const hz_grid* grid, const double* c_dev, const hz_params* p
     HZ_LAUNCHED();
     if (H->p.precision == HZ_C128) prepare_dinv_double(H);
     if (H->p.autotune) {
-      H->tuned_c64 = H->p.precision == HZ_C64;
       if (H->p.precision == HZ_C64) autotune_zblocks<float>(H);
       else autotune_zblocks<double>(H);
     }
@@ -2287,7 +2311,7 @@ extern "C" hz_status iofd_residual_static(hz_handle* H, int level, int op, int p
     // own over r, of at most 608 blocks per right-hand side, which always fits.
     const LevelView<double> lvd = view<double>(H, level);
     const long long blocks = !adj && precision == HZ_C64
-                                 ? fwd_blocks_c64(lv, nrhs)
+                                 ? fwd_blocks_c64(view<float>(H, level), nrhs)
                                  : resid_blocks(lv, level, nrhs, adj, lvd.zblock, lvd.zblock_f);
     const bool fused = blocks * nrhs <= kResidStaticPartials;
     static_assert(608 * kResidStaticMaxRhs <= kResidStaticPartials, "the norm pass fits");

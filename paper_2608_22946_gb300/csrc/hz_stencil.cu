@@ -351,7 +351,7 @@ void launch_stencil(const StencilCall<R>& c, int mode, int op, bool adjoint, cud
   if (!adjoint) {
     const int opk = fwd_opk(c, op);
     if constexpr (sizeof(R) == sizeof(float)) {
-      if (mode == M_AWIN || march::takes(mode, c.lv.nx, c.lv.ny, c.lv.nz, c.nrhs)) march::launch(c, mode, opk, s);
+      if (mode == M_AWIN || march::takes(c.lv, mode, opk == OPK_B, c.nrhs)) march::launch(c, mode, opk, s);
       else gather::launch_fwd_gather(c, mode, op, s);
     } else if (mode != M_AWIN && (c.lv.level > 0 || c.lv.N <= kSmallNodes)) {
       gather::launch_fwd_gather(c, mode, op, s);
@@ -387,7 +387,7 @@ void launch_stencil(const StencilCall<R>& c, int mode, int op, bool adjoint, cud
 long long stencil_blocks_per_rhs(int level, int nx, int ny, int nz, const int* plain_lo, const int* plain_hi,
                                  int nrhs, int zblock, int zblock_f) {
   if (level > 0 || (long long)nx * ny * nz <= kSmallNodes)
-    return gather::gather_blocks_per_rhs(nx, ny, nz, plain_lo, plain_hi, nrhs, zblock, zblock_f);
+    return gather::gather_blocks_per_rhs(false, nx, ny, nz, plain_lo, plain_hi, nrhs, zblock, zblock_f);
   const int zb = zblock > 0 ? zblock : choose_zblock(nx, ny, nz, nrhs);
   const FwdPlan p = plan_layout(nx, ny, nz, plain_lo, plain_hi, true, zb, zblock_f);
   return p.blocks();
@@ -411,12 +411,13 @@ long long adj_blocks_per_rhs(int nx, int ny, int nz, int nrhs, int zblock) {
 // saturating at 255.
 long long replay_fwd_layout(int level, int nx, int ny, int nz, const int* plo, const int* phi, int op, int nrhs,
                             int zblock, int zblock_f, unsigned char* counts, long long* blocks) {
-  // the single-precision launch has a layout of its own (march, small grids gather)
+  // the single-precision launches have layouts of their own (march, or gather where
+  // no mode or not every mode marches)
   long long single = march::replay_layout(nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f);
-  if (level == 0 && (long long)nx * ny * nz > kSmallNodes && !march::takes(M_J2, nx, ny, nz, 1))
-    single += gather::replay_gather_layout(nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f, nullptr, nullptr);
+  if (!march::takes(M_J2, true, nx, ny, nz, nrhs, plo, phi) || !march::takes(M_J2, false, nx, ny, nz, nrhs, plo, phi))
+    single += gather::replay_gather_layout(true, nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f, nullptr, nullptr);
   if (level > 0 || (long long)nx * ny * nz <= kSmallNodes)
-    return single + gather::replay_gather_layout(nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f, counts, blocks);
+    return single + gather::replay_gather_layout(false, nx, ny, nz, plo, phi, op, nrhs, zblock, zblock_f, counts, blocks);
   const bool ab = op == OP_AB;
   const int zb = zblock > 0 ? zblock : choose_zblock(nx, ny, nz, nrhs);
   const FwdPlan p = plan_layout(nx, ny, nz, plo, phi, ab, zb, zblock_f);

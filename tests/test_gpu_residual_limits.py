@@ -41,3 +41,22 @@ def test_residual_past_the_static_scratch(nz):
         assert torch.allclose(n2, ref2, rtol=ntol, atol=0)
         del x, g, r
     s.close()
+
+
+def test_complex128_residual_on_two_streams():
+    """105^3 in complex128: rectangle and PML frame are two launches, the frame on the
+    handle's second stream, and both add their block sums to the one static array."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2608_22946_gb300 as hz
+    w = W.layered_inclusion(n=104, n_pml=8, nsrc=1)
+    s = hz.Solver(w.n, w.n_pml, w.h, w.omega, w.c, max_nrhs=2)
+    gen = torch.Generator("cuda").manual_seed(5)
+    for _ in range(2):
+        x = torch.randn((2,) + s.level_shape[0], dtype=torch.complex128, device="cuda", generator=gen)
+        g = torch.randn(x.shape, dtype=torch.complex128, device="cuda", generator=gen)
+        r, n2 = s.residual_static(g, x)
+        ref = g - s.iofd_apply(x)
+        assert float(torch.linalg.vector_norm(r - ref) / torch.linalg.vector_norm(ref)) <= 3e-14
+        assert torch.allclose(n2, (ref.abs() ** 2).flatten(1).sum(1), rtol=3e-14, atol=0)
+    s.close()
