@@ -54,8 +54,7 @@ struct StencilCall {
   int zr0 = 0, zr1 = 0, xz0 = 0;
   long long xstride = 0, ystride = 0;
   int* err = nullptr;  // device flag set when a bounded wait of the kernel gave up
-  unsigned polls = 1u << 22;  // polls (64 ns apart) before such a wait gives up
-  unsigned extra = 0;         // > 0: the waits expect arrivals that never come (a test of that path)
+  unsigned extra = 0;  // > 0: such waits expect arrivals that never come, and end soon (a test of that path)
 };
 
 template <class R>

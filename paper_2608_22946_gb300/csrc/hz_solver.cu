@@ -177,7 +177,7 @@ struct hz_handle {
   double* bot_partial_f = nullptr;
   double* bot_partial_d = nullptr;
   unsigned bot_spins = 1u << 23, bot_extra = 0;
-  unsigned copy_polls = 1u << 22, copy_extra = 0;  // waits of the single-precision march
+  unsigned copy_extra = 0;  // the same for the waits of the single-precision march
   bool earlier_err = false;  // a wait of an asynchronous call gave up (set_aside_wait_err)
 };
 
@@ -574,7 +574,6 @@ StencilCall<R> call(hz_handle* H, int L, bool shifted, int nrhs) {
   c.fork = H->ev_fork;
   c.join = H->ev_join;
   c.err = H->bot_err;
-  c.polls = H->copy_polls;
   c.extra = H->copy_extra;
   return c;
 }
@@ -1815,10 +1814,7 @@ hz_status hz_create(const hz_grid* grid, const double* c_dev, const hz_params* p
         H->bot_spins = 4096;
       }
       const char* ct = std::getenv("HZ_COPY_TEST");  // makes every copy wait of the march run out (tests)
-      if (ct && ct[0] == '1') {
-        H->copy_extra = 1;
-        H->copy_polls = 4096;
-      }
+      H->copy_extra = ct && ct[0] == '1';
       if (H->coop_bottom) {
         H->bot_bar = H->al.get<unsigned>(2);
         H->bot_partial_f = H->al.get<double>(gather::bottom_partial_doubles<float>(max_nrhs));
