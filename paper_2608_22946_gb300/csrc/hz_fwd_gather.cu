@@ -767,7 +767,9 @@ static void launch_fwd_t(const StencilCall<R>& c, cudaStream_t s) {
   const LevelView<R>& L = c.lv;
   const FwdPlan p = plan_fwd(L, c.nrhs, OP);
   const int nblk_total = (int)p.blocks();
-  if (!p.split) {
+  // (single precision marches from the split's size on, but for the Jacobi map)
+  constexpr bool kSplits = OP == OP_AB && (sizeof(R) == sizeof(double) || MODE == M_J2);
+  if (!kSplits || !p.split) {
     TileMap tm;
     tm.ntx = p.TXT;
     tm.rx1 = L.nx - 1;
@@ -782,34 +784,36 @@ static void launch_fwd_t(const StencilCall<R>& c, cudaStream_t s) {
     k_fwd<R, MODE, OP, (OP == OP_Q) ? 0 : 2, CW><<<grid, dim3(TX, TY), 0, s>>>(c, p.zb, tm);
     return;
   }
-  TileMap ti;
-  ti.ox = p.frame.px0;
-  ti.oy = p.frame.py0;
-  ti.ntx = p.RW;
-  ti.rx1 = p.frame.px1;
-  ti.ry1 = p.frame.py1;
-  ti.bid_offset = 0;
-  ti.nblk_total = nblk_total;
-  TileMap tp = p.frame;
-  tp.bid_offset = p.RW * p.RH * p.nzb;
-  tp.nblk_total = nblk_total;
-  // the two launches are independent (disjoint outputs; a fused norm combines
-  // through its arrival counter): with a side stream they run concurrently
-  const bool fork = c.side && c.fork && c.join && tp.count > 0;
-  cudaStream_t s2 = fork ? c.side : s;
-  if (fork) {
-    cudaEventRecord(c.fork, s);
-    cudaStreamWaitEvent(s2, c.fork, 0);
-  }
-  count_launch();
-  k_fwd<R, MODE, OP, 0, CW><<<dim3(p.RW * c.nrhs, p.RH, p.nzb), dim3(TX, TY), 0, s>>>(c, p.zb, ti);
-  if (tp.count > 0) {
+  if constexpr (kSplits) {
+    TileMap ti;
+    ti.ox = p.frame.px0;
+    ti.oy = p.frame.py0;
+    ti.ntx = p.RW;
+    ti.rx1 = p.frame.px1;
+    ti.ry1 = p.frame.py1;
+    ti.bid_offset = 0;
+    ti.nblk_total = nblk_total;
+    TileMap tp = p.frame;
+    tp.bid_offset = p.RW * p.RH * p.nzb;
+    tp.nblk_total = nblk_total;
+    // the two launches are independent (disjoint outputs; a fused norm combines
+    // through its arrival counter): with a side stream they run concurrently
+    const bool fork = c.side && c.fork && c.join && tp.count > 0;
+    cudaStream_t s2 = fork ? c.side : s;
+    if (fork) {
+      cudaEventRecord(c.fork, s);
+      cudaStreamWaitEvent(s2, c.fork, 0);
+    }
     count_launch();
-    k_fwd<R, MODE, OP, 1, CW><<<dim3(tp.count * c.nrhs, 1, p.nzbf), dim3(TX, TY), 0, s2>>>(c, p.zbf, tp);
-  }
-  if (fork) {
-    cudaEventRecord(c.join, s2);
-    cudaStreamWaitEvent(s, c.join, 0);
+    k_fwd<R, MODE, OP, 0, CW><<<dim3(p.RW * c.nrhs, p.RH, p.nzb), dim3(TX, TY), 0, s>>>(c, p.zb, ti);
+    if (tp.count > 0) {
+      count_launch();
+      k_fwd<R, MODE, OP, 1, CW><<<dim3(tp.count * c.nrhs, 1, p.nzbf), dim3(TX, TY), 0, s2>>>(c, p.zbf, tp);
+    }
+    if (fork) {
+      cudaEventRecord(c.join, s2);
+      cudaStreamWaitEvent(s, c.join, 0);
+    }
   }
 }
 

@@ -31,11 +31,9 @@
 //  - blocks of 128 threads, three per SM (four with two right-hand sides): at 128
 //    registers the PML bodies spill, and every spill is a stall on a thrashed L1
 //    (289^3 A_h 147 us at four blocks, 138 at three).
-// Measured, in a CUDA graph, before / after (us): 289^3 A_h 194 / 136, residual
-// 278 / 183, J_2 290 / 242; its 2h level (145^3) A 36.5 / 26.7, B 36.4 / 27.5,
-// residual 58 / 45, J_2 50.2 / 42.2; 225^3 x 16 right-hand sides A_h 1191 / 967.
-// The core alone runs at 215 G nodes/s (4.3 TB/s of 20 B per node); PML rows at
-// about 80, bound by their 120 floating-point instructions per node.
+// Measured, in a CUDA graph, accumulation form / this (us): 289^3 A_h 194 / 135,
+// residual 278 / 182, J_2 290 / 224; its 2h level (145^3) A 36.5 / 26.7, B 36.4 / 27.6,
+// residual 58 / 46, J_2 50.2 / 43.3; 225^3 x 16 right-hand sides A_h 1191 / 972.
 #pragma once
 
 #include <cuda.h>
@@ -553,17 +551,13 @@ __device__ __forceinline__ void tile_body(const StencilCall<float>& a, unsigned 
       float2 v[NPY + 2][NPX + 2], hx[NPY + 2][NPX];
 #pragma unroll
       for (int q = 0; q < NPY + 2; ++q) {
-        if constexpr (NPX == 2) {
-          const float4 u0 = *reinterpret_cast<const float4*>(P + q * PW);
-          const float4 u1 = *reinterpret_cast<const float4*>(P + q * PW + 2);
-          v[q][0] = make_float2(u0.x, u0.y);
-          v[q][1] = make_float2(u0.z, u0.w);
-          v[q][2] = make_float2(u1.x, u1.y);
-          v[q][3] = make_float2(u1.z, u1.w);
-        } else {
-#pragma unroll
-          for (int i = 0; i < NPX + 2; ++i) v[q][i] = ldf2(P + q * PW + i);
-        }
+        static_assert(NPX == 2, "a row's values come as two 128-bit loads");
+        const float4 u0 = *reinterpret_cast<const float4*>(P + q * PW);
+        const float4 u1 = *reinterpret_cast<const float4*>(P + q * PW + 2);
+        v[q][0] = make_float2(u0.x, u0.y);
+        v[q][1] = make_float2(u0.z, u0.w);
+        v[q][2] = make_float2(u1.x, u1.y);
+        v[q][3] = make_float2(u1.z, u1.w);
 #pragma unroll
         for (int i = 0; i < NPX; ++i) hx[q][i] = add2(v[q][i], v[q][i + 2]);
       }
@@ -813,7 +807,7 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
 
   // element a of the warp's first halo row in plane 0 (right-hand side rhs0); the
   // rows' places in a stage
-  const int a0 = (mp.sx + (row0 + NPY * ty) * nx + x0 - 1) & 1;
+  const int a0 = (int)((unsigned)mp.sx + (unsigned)(row0 + NPY * ty) * (unsigned)nx + (unsigned)(x0 - 1)) & 1;
   unsigned xo[NPY + 2];
 #pragma unroll
   for (int q = 0; q < NPY + 2; ++q) xo[q] = ((NPY * ty + q) & 1) * SM::half + ((NPY * ty + q) >> 1) * kRowB + 16 * lane;
@@ -823,8 +817,8 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
   // Jacobi map: y1 / omega = D^-1 g of a landed plane, in place
   auto transform = [&](int k, int st) {
     const unsigned xb = sb + st * SM::stage;
-    const unsigned px = (unsigned)(mp.sx + (row0 + k * L.ny) * nx + x0 - 1),
-                   pd = (unsigned)((rowd + k * L.ny) * nx + x0 - 1);
+    const unsigned px = (unsigned)mp.sx + (unsigned)(row0 + k * L.ny) * (unsigned)nx + (unsigned)(x0 - 1),
+                   pd = (unsigned)(rowd + k * L.ny) * (unsigned)nx + (unsigned)(x0 - 1);
     for (int row = ty; row < XR; row += NT / 32) {
       const unsigned ro = xb + (row & 1) * SM::half + (row >> 1) * kRowB + 8 * lane;
       const unsigned ax = 8 * ((px + row * nx) & 1), ad = 8 * ((pd + row * nx) & 1);
@@ -974,7 +968,7 @@ __device__ __forceinline__ void core_body(const StencilCall<float>& a, const Map
               }
             } else if constexpr (J2) {
               const int sp = st == 0 ? NSTG - 1 : st - 1;
-              const unsigned di = (unsigned)((rowd + (k - 1) * L.ny + NPY * ty + j + 1) * nx + x0 - 1) & 1;
+              const unsigned di = ((unsigned)(rowd + (k - 1) * L.ny + NPY * ty + j + 1) * (unsigned)nx + (unsigned)(x0 - 1)) & 1;
               const float2 d = lds64(sb + sp * SM::stage + SM::o_d + xo[j + 1] + 8 * (di + 1 + i));
               out = jacobi2(om, d, oc, h);
               if (a.base) {
