@@ -102,8 +102,8 @@ void launch_block_gram(const BlockCols& X, const BlockCols& Y, double* partial, 
 template <class R>
 void launch_block_update(const BlockCols& X, cx<R>* Y, int q, const double* C, double beta, cudaStream_t s);
 void block_init_attrs();
-// Grids of at most this many nodes run as many small blocks (8 x 8 tiles, two
-// planes), in the gather form on every level, forward and adjoint: see k_fwd_small.
+// Grids of at most this many nodes run as many small blocks (8 x 8 tiles, two planes
+// or more as right-hand sides supply blocks), in the gather form on every level, forward and adjoint: see k_fwd_small.
 // Above the line, B apply / residual / J_2 in a CUDA graph (us), 256-thread tiles
 // against 8 x 8 tiles of 2 and of 4 planes: complex64 53^3 5.5 / 14.4 / 6.5, 5.3 /
 // 18.5 / 8.2, 5.9 / 16.5 / 6.8; 73^3 8.1 / 18.6 / 10.1, 11.0 / 31.1 / 15.1, 10.6 /
